@@ -118,7 +118,33 @@ mosaic_status gemm_u32(int variant, Carve &cv, const uint32_t *A, int64_t sai, i
     return s;
 }
 
-size_t ws_chains(int64_t n_pad, const mosaic_params *p) {
+// C = (Cin ? Cin : 0) + A B for a B given K x N (K down its rows), on the
+// tensor cores: A's digit planes and those of B's transpose are written to
+// `cv`.  False if the variant or the room does not allow it (nothing is
+// enqueued then).
+bool gemm_kn_tc_fits(int variant, const Carve &cv, int64_t M, int64_t N, int64_t K) {
+    const bool want_tc = variant == MOSAIC_GEMM_TC || (variant == MOSAIC_GEMM_AUTO && tc_available());
+    const int64_t Kp = (K + 7) / 8 * 8;
+    return want_tc && K > 0 && cv.used + up(8 * (size_t)(M * Kp)) + up(8 * (size_t)(N * Kp)) <= cv.cap;
+}
+mosaic_status gemm_kn_tc(Carve &cv, const uint32_t *A, int64_t lda, const uint32_t *B, int64_t ldb, uint32_t *C,
+                         int64_t ldc, const uint32_t *Cin, int64_t ldcin, int64_t M, int64_t N, int64_t K,
+                         cudaStream_t st) {
+    const int64_t Kp = (K + 7) / 8 * 8;
+    const size_t mark = cv.used;
+    uint16_t *Ap = cv.take<uint16_t>((size_t)(4 * M * Kp));
+    uint16_t *Bp = cv.take<uint16_t>((size_t)(4 * N * Kp));
+    if (!Ap || !Bp) return MOSAIC_ERR_WORKSPACE;
+    MOSAIC_TRY(digit_split(A, lda, M, K, Ap, Kp, M * Kp, st));
+    MOSAIC_TRY(digit_split_t(B, ldb, K, N, Bp, Kp, N * Kp, st));
+    const mosaic_status s = ring_gemm_tc_planes(Ap, Kp, M * Kp, Bp, Kp, N * Kp, C, ldc, Cin, ldcin, 1, M, N, K, st);
+    cv.used = mark;
+    return s;
+}
+
+// Minimum workspace of the chains (M_i and N_i) and the extra room that lets
+// their products run on the tensor cores (both operands' digit planes).
+size_t ws_chains_min(int64_t n_pad, const mosaic_params *p) {
     size_t s = 0;
     int64_t prev = n_pad;
     for (uint32_t i = 1; i <= p->d; i++) {
@@ -127,6 +153,15 @@ size_t ws_chains(int64_t n_pad, const mosaic_params *p) {
         prev = ri;
     }
     return s;
+}
+size_t ws_chains(int64_t n_pad, const mosaic_params *p) {
+    size_t planes = 0;
+    for (uint32_t i = 2; i <= p->d; i++) {
+        const int64_t Kp = ((int64_t)p->r[i - 2] + 7) / 8 * 8;
+        const size_t s = up(8 * (size_t)(p->r[i - 1] * Kp)) + up(8 * (size_t)(n_pad * Kp));
+        planes = s > planes ? s : planes;
+    }
+    return ws_chains_min(n_pad, p) + planes;
 }
 int64_t sum_r(const mosaic_params *p);
 // Minimum workspaces (CUDA-core products) and the extra room that lets the
@@ -444,7 +479,7 @@ mosaic_status mosaic_mask_chains(const mosaic_params *p, const mosaic_key *key, 
     if (!key) return MOSAIC_ERR_ARG;
     if (!npad_ok(n_pad)) return MOSAIC_ERR_SHAPE;
     if (!P || !C || !CT) return MOSAIC_ERR_ARG;
-    if (ws_bytes < ws_chains(n_pad, p)) return MOSAIC_ERR_WORKSPACE;
+    if (ws_bytes < ws_chains_min(n_pad, p)) return MOSAIC_ERR_WORKSPACE;
     cudaStream_t st = as_stream(stream);
     const Key k = to_key(key);
     const int R = (int)p->rounds;
@@ -453,6 +488,13 @@ mosaic_status mosaic_mask_chains(const mosaic_params *p, const mosaic_key *key, 
     // Level 1: M_1 (r_1 x n_pad) is P_1; N_1 (n_pad x r_1) is C_1.
     MOSAIC_TRY(prg_uniform(k, tag_of(MOSAIC_TAG_M, 1), chain_id, R, p->r[0], n_pad, P, n_pad, st));
     MOSAIC_TRY(prg_uniform(k, tag_of(MOSAIC_TAG_N, 1), chain_id, R, n_pad, p->r[0], C, Sr, st));
+    // Level i: P_i = M_i P_{i-1} (r_i x n_pad) and C_i = C_{i-1} N_i (n_pad x r_i),
+    // both with K = r_{i-1} down the rows of the second factor.  On the tensor
+    // cores when the workspace has room for the digit planes (the CUDA-core
+    // product reads the second factor strided).  Chains and Init W of a
+    // 4096 x 4096 matrix: 3.78 -> 2.22 ms, of which the four CUDA-core chain
+    // products (18.4 G MACs, 10 T MAC/s) were 1.88 ms.
+    Carve mn{cv.base, cv.cap, cv.used + ws_chains_min(n_pad, p)};   // planes, behind every M_i and N_i
     for (uint32_t i = 2; i <= p->d; i++) {
         const int64_t ri = p->r[i - 1], rp = p->r[i - 2];
         const int64_t oi = off_r(p, i), op = off_r(p, i - 1);
@@ -461,12 +503,18 @@ mosaic_status mosaic_mask_chains(const mosaic_params *p, const mosaic_key *key, 
         if (!Mi || !Ni) return MOSAIC_ERR_WORKSPACE;
         MOSAIC_TRY(prg_uniform(k, tag_of(MOSAIC_TAG_M, i), chain_id, R, ri, rp, Mi, rp, st));
         MOSAIC_TRY(prg_uniform(k, tag_of(MOSAIC_TAG_N, i), chain_id, R, rp, ri, Ni, ri, st));
-        // P_i = M_i P_{i-1}:  C(a, c) = sum_b M_i[a][b] P_{i-1}[b][c]
-        MOSAIC_TRY(ring_gemm_imad(Mi, rp, 1, P + op * n_pad, 1, n_pad, P + oi * n_pad, n_pad,
-                                  nullptr, 0, 1, ri, n_pad, rp, st));
-        // C_i = C_{i-1} N_i:  C(c, b) = sum_a C_{i-1}[c][a] N_i[a][b]
-        MOSAIC_TRY(ring_gemm_imad(C + op, Sr, 1, Ni, 1, ri, C + oi, Sr, nullptr, 0, 1, n_pad, ri,
-                                  rp, st));
+        const uint32_t *Pp = P + op * n_pad, *Cp = C + op;
+        uint32_t *Pi = P + oi * n_pad, *Ci = C + oi;
+        if (gemm_kn_tc_fits(MOSAIC_GEMM_AUTO, mn, ri, n_pad, rp)) {
+            MOSAIC_TRY(gemm_kn_tc(mn, Mi, rp, Pp, n_pad, Pi, n_pad, nullptr, 0, ri, n_pad, rp, st));
+        } else {
+            MOSAIC_TRY(ring_gemm_imad(Mi, rp, 1, Pp, 1, n_pad, Pi, n_pad, nullptr, 0, 1, ri, n_pad, rp, st));
+        }
+        if (gemm_kn_tc_fits(MOSAIC_GEMM_AUTO, mn, n_pad, ri, rp)) {
+            MOSAIC_TRY(gemm_kn_tc(mn, Cp, Sr, Ni, ri, Ci, Sr, nullptr, 0, n_pad, ri, rp, st));
+        } else {
+            MOSAIC_TRY(ring_gemm_imad(Cp, Sr, 1, Ni, 1, ri, Ci, Sr, nullptr, 0, 1, n_pad, ri, rp, st));
+        }
     }
     return transpose_u32(C, Sr, n_pad, Sr, CT, n_pad, st);
 }
@@ -501,9 +549,8 @@ mosaic_status mosaic_mask_weight(const mosaic_params *p, const mosaic_key *key, 
     const int32_t qmax = mosaic_qmax(n_pad, p->qbits);
     MOSAIC_TRY(fwht_encode(W, ldw, m, n, n_pad, sign_words, 1, 1, nullptr, qmax, nullptr, 0, Wp,
                            n_pad, s_w, nullptr, st));
-    // E_w and W_hat + E_w.
-    MOSAIC_TRY(prg_gaussian(k, tag_of(MOSAIC_TAG_EW, 0), matrix_id, R, p->sigma, m * n_pad, WE, st));
-    MOSAIC_TRY(add_u32(Wp, n_pad, WE, n_pad, WE, n_pad, m, n_pad, st));
+    // W_hat + E_w, added as E_w is drawn.
+    MOSAIC_TRY(prg_gaussian(k, tag_of(MOSAIC_TAG_EW, 0), matrix_id, R, p->sigma, m * n_pad, WE, st, nullptr, Wp));
     // J_i = (W_hat + E_w) C_i for all i at once: J = WE CT^T (m x Sr); with
     // act_nested = 0 only J_1 (the first r_1 columns) is used and computed.
     const int64_t nJ = p->act_nested ? Sr : (int64_t)p->r[0];
@@ -521,11 +568,14 @@ mosaic_status mosaic_mask_weight(const mosaic_params *p, const mosaic_key *key, 
     }
     // W' = (W_hat + E_w) + L P_d + sum_i S_{i+1} P_i.  With room in the
     // workspace (the J product's digit planes are released by now), L P_d
-    // runs against P_d^T (K-major, so the tensor cores can take it) and the
-    // sparse terms run on the tiled gather with the rows of P^T as its staged
-    // rows; otherwise the product reads P_d strided and a plain row gather
-    // reads P.
-    {
+    // runs on the tensor cores from the digit planes of P_d^T, or against
+    // P_d^T itself (K-major, for the other variants and for a few rows), and
+    // the sparse terms run on the tiled gather with the rows of P^T as its
+    // staged rows; otherwise the product reads P_d strided and a plain row
+    // gather reads P.
+    if (m > kSkinnyMaxM && gemm_kn_tc_fits(variant, cv, m, n_pad, rd)) {
+        MOSAIC_TRY(gemm_kn_tc(cv, L, rd, P + od * n_pad, n_pad, Wp, n_pad, WE, n_pad, m, n_pad, rd, st));
+    } else {
         const size_t mark = cv.used;
         uint32_t *PdT = cv.take<uint32_t>((size_t)(n_pad * rd));
         if (PdT) {

@@ -138,9 +138,10 @@ inline int grid_for(int64_t items, int threads) {
 mosaic_status prg_uniform(const Key &key, uint32_t tag, uint64_t sid, int rounds, int64_t rows,
                           int64_t cols, uint32_t *out, int64_t ldo, cudaStream_t st,
                           const uint64_t *sid_dev = nullptr);
-// Discrete Gaussian elements.
+// Discrete Gaussian elements; with `add`, out = add + the samples.
 mosaic_status prg_gaussian(const Key &key, uint32_t tag, uint64_t sid, int rounds, float sigma,
-                           int64_t count, uint32_t *out, cudaStream_t st, const uint64_t *sid_dev = nullptr);
+                           int64_t count, uint32_t *out, cudaStream_t st, const uint64_t *sid_dev = nullptr,
+                           const uint32_t *add = nullptr);
 // Sparse rows.
 // All draws of an Init X call in one launch: R (l x rd, and its digit planes
 // [4][l][Kp] when Rp is not null), nlev <= 2 sparse lists (l rows each) and
@@ -177,6 +178,10 @@ mosaic_status ring_gemm_imad(const uint32_t *A, int64_t sai, int64_t sak, const 
 // Digit planes.
 mosaic_status digit_split(const uint32_t *a, int64_t lda, int64_t rows, int64_t cols,
                           uint16_t *planes, int64_t ldp, int64_t plane_stride, cudaStream_t st);
+// Digit planes of a's transpose: planes[d][c][k] = digit d of a[k][c] (ldp and
+// plane_stride multiples of 4, planes 8-byte aligned).
+mosaic_status digit_split_t(const uint32_t *a, int64_t lda, int64_t rows, int64_t cols, uint16_t *planes,
+                            int64_t ldp, int64_t plane_stride, cudaStream_t st);
 
 // Tensor-core ring GEMM from planes (NT, K-major planes); C = (Cin?) + sgn * A B^T.
 mosaic_status ring_gemm_tc_planes(const uint16_t *Ap, int64_t ldpa, int64_t a_plane,
@@ -313,9 +318,7 @@ mosaic_status unmask_decode(const uint32_t *Z, int64_t ldz, int64_t seg_off, int
 mosaic_status sparse_rowgather(const uint32_t *P, int64_t ldp, const SparseLevel *lev, int nlev,
                                int64_t m, int64_t ncols, const uint32_t *a, int64_t lda,
                                uint32_t *out, int64_t ldo, cudaStream_t st);
-// Elementwise and layout helpers.
-mosaic_status add_u32(const uint32_t *a, int64_t lda, const uint32_t *b, int64_t ldb, uint32_t *out,
-                      int64_t ldo, int64_t rows, int64_t cols, cudaStream_t st);
+// Layout helper.
 mosaic_status transpose_u32(const uint32_t *a, int64_t lda, int64_t rows, int64_t cols, uint32_t *out,
                             int64_t ldo, cudaStream_t st);
 

@@ -68,10 +68,11 @@ struct GaussTable {
 // two (largest first) while the entry just below pos + step is still <= u.
 // Samples [8 first, ...) of the Gaussian stream, `stride` threads; st = the
 // table in shared memory (tab.n entries), top = largest power of two <= n.
-// tab.n == 0 writes zeros (sigma = 0).
+// tab.n == 0 writes zeros (sigma = 0).  With `add`, out = add + the samples.
 __device__ __forceinline__ void gaussian_body(const Key &key, uint32_t tag, uint32_t sid_lo, uint32_t sid_hi,
                                               int rounds, const unsigned long long *st, int n, int bound, int top,
-                                              int64_t count, uint32_t *out, int64_t first, int64_t stride) {
+                                              int64_t count, uint32_t *out, int64_t first, int64_t stride,
+                                              const uint32_t *add) {
     const int64_t nblk = (count + 7) / 8;
     for (int64_t b = first; b < nblk; b += stride) {
         uint32_t res[8];
@@ -92,6 +93,17 @@ __device__ __forceinline__ void gaussian_body(const Key &key, uint32_t tag, uint
             }
         }
         const int64_t e0 = b * 8;
+        if (add) {
+            if (e0 + 8 <= count && ((reinterpret_cast<uintptr_t>(add + e0) & 15u) == 0)) {
+                const uint4 x = reinterpret_cast<const uint4 *>(add + e0)[0], y = reinterpret_cast<const uint4 *>(add + e0)[1];
+                res[0] += x.x; res[1] += x.y; res[2] += x.z; res[3] += x.w;
+                res[4] += y.x; res[5] += y.y; res[6] += y.z; res[7] += y.w;
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; i++)
+                    if (e0 + i < count) res[i] += add[e0 + i];
+            }
+        }
         if (e0 + 8 <= count && ((reinterpret_cast<uintptr_t>(out + e0) & 15u) == 0)) {
             reinterpret_cast<uint4 *>(out + e0)[0] = make_uint4(res[0], res[1], res[2], res[3]);
             reinterpret_cast<uint4 *>(out + e0)[1] = make_uint4(res[4], res[5], res[6], res[7]);
@@ -108,14 +120,14 @@ __device__ __forceinline__ int pow2_floor(int n) {
 }
 
 __global__ void gaussian_kernel(Key key, uint32_t tag, uint64_t sid, const uint64_t *sid_dev, int rounds,
-                                GaussTable tab, int64_t count, uint32_t *out) {
+                                GaussTable tab, int64_t count, uint32_t *out, const uint32_t *add) {
     __shared__ unsigned long long st[2 * kMaxGaussBound + 1];
     uint32_t sid_lo, sid_hi;
     stream_id(sid, sid_dev, sid_lo, sid_hi);
     for (int i = threadIdx.x; i < tab.n; i += blockDim.x) st[i] = tab.t[i];
     __syncthreads();
     gaussian_body(key, tag, sid_lo, sid_hi, rounds, st, tab.n, tab.bound, pow2_floor(tab.n), count, out,
-                  blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
+                  blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x, add);
 }
 
 // One warp per sparse row; the row's window starts at block row * 4096.
@@ -261,7 +273,7 @@ __global__ void __launch_bounds__(kDrawThreads) initx_draw_kernel(InitxDraws a) 
     __syncthreads();
     gaussian_body(a.key, a.tagE, sid_lo, sid_hi, a.rounds, st, a.tab.n, a.tab.bound,
                   a.tab.n ? pow2_floor(a.tab.n) : 0, a.ecount, a.E, (int64_t)blk * kDrawThreads + threadIdx.x,
-                  (int64_t)a.nbG * kDrawThreads);
+                  (int64_t)a.nbG * kDrawThreads, nullptr);
 }
 
 // Sampler grids: one thread per ChaCha block, up to 152 x 64 blocks.
@@ -308,9 +320,13 @@ mosaic_status prg_uniform(const Key &key, uint32_t tag, uint64_t sid, int rounds
 }
 
 mosaic_status prg_gaussian(const Key &key, uint32_t tag, uint64_t sid, int rounds, float sigma,
-                           int64_t count, uint32_t *out, cudaStream_t st, const uint64_t *sid_dev) {
+                           int64_t count, uint32_t *out, cudaStream_t st, const uint64_t *sid_dev,
+                           const uint32_t *add) {
     if (count == 0) return MOSAIC_OK;
     if (sigma == 0.0f) {
+        if (add)
+            return cudaMemcpyAsync(out, add, sizeof(uint32_t) * (size_t)count, cudaMemcpyDeviceToDevice, st) == cudaSuccess
+                       ? MOSAIC_OK : MOSAIC_ERR_CUDA;
         return cudaMemsetAsync(out, 0, sizeof(uint32_t) * (size_t)count, st) == cudaSuccess
                    ? MOSAIC_OK : MOSAIC_ERR_CUDA;
     }
@@ -321,7 +337,7 @@ mosaic_status prg_gaussian(const Key &key, uint32_t tag, uint64_t sid, int round
     {
         KernelSpan span("prg_gaussian", st);
         gaussian_kernel<<<prg_blocks(nblk, kThreads), kThreads, 0, st>>>(
-            key, tag, sid, sid_dev, rounds, tab, count, out);
+            key, tag, sid, sid_dev, rounds, tab, count, out, add);
     }
     return launch_status();
 }

@@ -732,16 +732,6 @@ __global__ void rowgather_kernel(const uint32_t *P, int64_t ldp, SparseLevel l0,
     out[j * ldo + c] = acc;
 }
 
-__global__ void add_kernel(const uint32_t *a, int64_t lda, const uint32_t *b, int64_t ldb,
-                           uint32_t *out, int64_t ldo, int64_t rows, int64_t cols) {
-    const int64_t total = rows * cols;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = i / cols, c = i - r * cols;
-        out[r * ldo + c] = a[r * lda + c] + b[r * ldb + c];
-    }
-}
-
 __global__ void transpose_kernel(const uint32_t *a, int64_t lda, int64_t rows, int64_t cols,
                                  uint32_t *out, int64_t ldo) {
     __shared__ uint32_t tile[32][33];
@@ -789,6 +779,46 @@ __global__ void digit_split_kernel(const uint32_t *a, int64_t lda, int64_t rows,
     }
 }
 
+// Digit planes of the TRANSPOSE of a (rows x cols): planes[d][c][k] = digit d
+// of a[k][c], k < rows, for products whose K runs down the rows of a.  Bound
+// by memory traffic (4 bytes read and 8 written an element); block (x, y)
+// moves 64 rows x 32 columns through shared memory so that both sides go out
+// in whole 128-byte lines: rows of 32 words in, 64 K of one column and plane
+// out.  One pass instead of a transpose (8 bytes an element) and a split.
+constexpr int kStRows = 64, kStCols = 32;
+__global__ void __launch_bounds__(256) digit_split_t_kernel(const uint32_t *a, int64_t lda, int64_t rows,
+                                                            int64_t cols, uint16_t *planes, int64_t ldp,
+                                                            int64_t plane_stride) {
+    __shared__ uint32_t t[kStRows][kStCols + 1];
+    const int64_t k0 = (int64_t)blockIdx.y * kStRows, c0 = (int64_t)blockIdx.x * kStCols;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = ty; k < kStRows; k += 8) {
+        const int64_t gk = k0 + k, gc = c0 + tx;
+        t[k][tx] = (gk < rows && gc < cols) ? a[gk * lda + gc] : 0u;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = threadIdx.x; i < kStCols * (kStRows / 4); i += 256) {
+        const int q = i & 15, c = i >> 4;   // K values 4 q .. 4 q + 3 of column c
+        if (c0 + c >= cols) continue;
+        uint32_t v[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) v[j] = t[4 * q + j][c];
+        uint16_t *dst = planes + (c0 + c) * ldp + k0 + 4 * q;
+        if (k0 + 4 * q + 4 <= rows) {
+#pragma unroll
+            for (int d = 0; d < 4; d++)
+                *reinterpret_cast<uint2 *>(dst + d * plane_stride) =
+                    make_uint2(digit_bits(v[0], d) | (digit_bits(v[1], d) << 16),
+                               digit_bits(v[2], d) | (digit_bits(v[3], d) << 16));
+        } else {
+            for (int j = 0; j < 4 && k0 + 4 * q + j < rows; j++)
+#pragma unroll
+                for (int d = 0; d < 4; d++) dst[d * plane_stride + j] = (uint16_t)digit_bits(v[j], d);
+        }
+    }
+}
 
 // Tile images for the tiled gather: image t holds rows 32 t .. 32 t + 31 of
 // the segment src[:, col0 .. col0 + r) exactly as pgather_kernel stages them
@@ -1115,16 +1145,6 @@ mosaic_status sparse_rowgather(const uint32_t *P, int64_t ldp, const SparseLevel
     return launch_status();
 }
 
-mosaic_status add_u32(const uint32_t *a, int64_t lda, const uint32_t *b, int64_t ldb, uint32_t *out,
-                      int64_t ldo, int64_t rows, int64_t cols, cudaStream_t st) {
-    if (rows == 0 || cols == 0) return MOSAIC_OK;
-    {
-        KernelSpan span("ring_add", st);
-        add_kernel<<<grid_for(rows * cols, 256), 256, 0, st>>>(a, lda, b, ldb, out, ldo, rows, cols);
-    }
-    return launch_status();
-}
-
 mosaic_status transpose_u32(const uint32_t *a, int64_t lda, int64_t rows, int64_t cols, uint32_t *out,
                             int64_t ldo, cudaStream_t st) {
     if (rows == 0 || cols == 0) return MOSAIC_OK;
@@ -1147,6 +1167,20 @@ mosaic_status digit_split(const uint32_t *a, int64_t lda, int64_t rows, int64_t 
         KernelSpan span("digit_split", st);
         digit_split_kernel<<<grid_for(rows * ((cols + 3) / 4), 256), 256, 0, st>>>(
             a, lda, rows, cols, planes, ldp, plane_stride, vec);
+    }
+    return launch_status();
+}
+
+mosaic_status digit_split_t(const uint32_t *a, int64_t lda, int64_t rows, int64_t cols, uint16_t *planes,
+                            int64_t ldp, int64_t plane_stride, cudaStream_t st) {
+    if (rows == 0 || cols == 0) return MOSAIC_OK;
+    if (ldp % 4 || plane_stride % 4 || (reinterpret_cast<uintptr_t>(planes) & 7u)) return MOSAIC_ERR_ALIGN;
+    const int64_t gx = (cols + kStCols - 1) / kStCols, gy = (rows + kStRows - 1) / kStRows;
+    if (gx > 0x7fffffff || gy > 65535) return MOSAIC_ERR_SHAPE;
+    {
+        KernelSpan span("digit_split_t", st);
+        digit_split_t_kernel<<<dim3((unsigned)gx, (unsigned)gy), 256, 0, st>>>(a, lda, rows, cols, planes, ldp,
+                                                                              plane_stride);
     }
     return launch_status();
 }

@@ -67,3 +67,30 @@ def test_freivalds_matches_oracle_and_detects(m, n, l, k):
         Zq[0, m] += 1
         bad, n_bad = layer.freivalds_check(Zq, Xp)
         assert _host(n_bad)[0] == 0
+
+
+# Both token groupings (below and from 76 tokens), every cluster split, ragged
+# groups, all vector-count steps, columns fewer than a share, and strides that
+# forbid 16-byte loads of one or both operands.
+@pytest.mark.parametrize("l,m,n,k,dz,dx", [
+    (1, 17, 4, 16, 0, 0), (1, 4096, 8192, 1, 0, 0), (5, 100, 64, 2, 3, 0), (75, 333, 257, 3, 1, 1),
+    (76, 64, 32, 4, 0, 4), (77, 1000, 96, 5, 5, 0), (303, 130, 131, 8, 2, 2), (610, 40, 64, 9, 0, 0),
+    (1300, 52, 36, 16, 4, 0)])
+def test_check_counts_differing_vectors(l, m, n, k, dz, dx):
+    from paper_2607_29221_gb300 import mosaic as M
+    rng = np.random.default_rng(l * 31 + k)
+    u32 = lambda *s: rng.integers(0, 1 << 32, s, dtype=np.uint32)
+    a, Yc, Z, X = u32(k, m), u32(k, n), u32(l, m + dz), u32(l, n + dx)
+    a[:, :k] = np.eye(k, dtype=np.uint32)
+    # Honest answers: column v < k is chosen so that vector v agrees; then a third of the tokens is tampered with.
+    Z[:, :k] = X[:, :n] @ Yc.T - Z[:, k:m] @ a[:, k:].T
+    off = rng.integers(0, l, l // 3 + 1)
+    Z[off, rng.integers(0, m, len(off))] += np.uint32(1 << 31)
+    want = np.count_nonzero(Z[:, :m] @ a.T != X[:, :n] @ Yc.T, axis=1)
+    dev = lambda x: torch.from_numpy(x.view(np.int32)).cuda()
+    bad = torch.full((l,), -1, dtype=torch.int32, device="cuda")
+    n_bad = torch.full((1,), 7, dtype=torch.int32, device="cuda")
+    ws = torch.empty(M.mosaic_workspace_bytes(M.OP_FREIVALDS_CHECK, k, 0, l), dtype=torch.uint8, device="cuda")
+    M.mosaic_freivalds_check(k, dev(a), dev(Yc), m, n, l, dev(Z), m + dz, dev(X), n + dx, bad, n_bad, ws)
+    assert np.array_equal(_host(bad), want.astype(np.uint32))
+    assert _host(n_bad)[0] == 7 + np.count_nonzero(want)

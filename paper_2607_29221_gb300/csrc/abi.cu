@@ -841,6 +841,14 @@ mosaic_status unmask_impl(const mosaic_params *p, int64_t l, int64_t m, const ui
         lev[i - 1] = SparseLevel{S_idx + soff, S_val + soff, (int)t, m + off_r(p, i), ri};
         soff += m * t;
     }
+    // Up to 16 tokens everything runs in one launch, which reads L and the S
+    // lists once (70B gate+up at one token: 80 us as a product and two gathers).
+    if (want_tc && unmask_few_ok(l, m, rd, (int)d - 1, lev))
+        return unmask_few(l, m, Z, ldz, m + od, rd, K_tm, L, (int)d - 1, lev, s_w, s_x, bias, Y, Yhat, ldy, st);
+    const int64_t Kp = kpad8(rd);
+    const bool tc_planes = Lp && want_tc && !skinny_ok(Qd, ldz, L, rd, l, rd) && ldz % 4 == 0 && aligned16(Qd) &&
+                           cv.used + up(8 * (size_t)(l * Kp)) <= cv.cap;
+    uint16_t *Qp = tc_planes ? cv.take<uint16_t>((size_t)(4 * l * Kp)) : nullptr;
     // With room in the workspace, the gathers stage Q_i from tile images made
     // here, in the same launch that splits Q_d into digit planes.
     int nimg = 0;

@@ -314,6 +314,15 @@ mosaic_status unmask_decode(const uint32_t *Z, int64_t ldz, int64_t seg_off, int
                             const uint32_t *tmp, int64_t ldt, const float *s_w, const float *s_x,
                             const float *bias, float *Y, uint32_t *Yhat, int64_t ldy,
                             cudaStream_t st, bool folded = false);
+// The whole unmask and decode of at most 16 tokens in one launch (lev[i].off:
+// first column of Q_i in Z, dcol: of Q_d); unmask_few_ok() tells whether the
+// ranks leave room to stage Q in shared memory.
+constexpr size_t kUnmaskFewSmem = 224 * 1024;
+bool unmask_few_ok(int64_t l, int64_t m, int64_t rd, int nlev, const SparseLevel *lev);
+mosaic_status unmask_few(int64_t l, int64_t m, const uint32_t *Z, int64_t ldz, int64_t dcol, int64_t rd,
+                         const uint32_t *K_tm, const uint32_t *L, int nlev, const SparseLevel *lev, const float *s_w,
+                         const float *s_x, const float *bias, float *Y, uint32_t *Yhat, int64_t ldy,
+                         cudaStream_t st);
 // out[j][c] = a[j][c] + sum_lev sum_q val[j][q] * P[(row_off_lev + idx[j][q]) * ldp + c]
 mosaic_status sparse_rowgather(const uint32_t *P, int64_t ldp, const SparseLevel *lev, int nlev,
                                int64_t m, int64_t ncols, const uint32_t *a, int64_t lda,

@@ -526,3 +526,15 @@ def test_rotation_and_encode_streamed_rows(n_pad):
                 rebuilt = sum(pl[i] << (8 * i) for i in range(4)) % (1 << 32)
                 assert np.array_equal(rebuilt.astype(np.uint32), got)
     M.mosaic_device_status()
+
+
+# The one-launch unmask of up to 16 tokens: every token-count step, ranks and weights that are no
+# multiples of 4, 32 or a warp's prefetch (96 pairs, 768 words), one to three levels, fewer rows than
+# one block's warps, and ranks too large to stage (16 x 3900 words: the general path).
+@pytest.mark.parametrize("d,r,t,m,l", [
+    (3, (100, 70, 37), (9, 7), 131, 3), (3, (300, 260, 900), (110, 100), 65, 9), (1, (96,), (), 40, 7),
+    (2, (1030, 20), (4,), 3, 16), (3, (1536, 1024, 652), (80, 80), 700, 8), (3, (96, 64, 40), (6, 5), 1, 2),
+    (3, (2000, 1500, 400), (12, 8), 33, 16), (3, (1537, 33, 5), (100, 3), 90, 1)])
+def test_unmask_of_few_tokens(d, r, t, m, l):
+    g, ref, op, m, l = _run_layer(d, r, t, m=m, n=200, l=l, variant=M_().GEMM_AUTO)
+    _check_layer(g, ref, op, m, l)

@@ -255,12 +255,12 @@ int mosaic_gemm_variant_available(int variant);
  * IMAD needs no workspace.  TC requires lda, ldb multiples of 4 and 16-byte
  * aligned A, B (MOSAIC_ERR_ALIGN otherwise; AUTO then runs IMAD).  With
  * 1 <= M <= MOSAIC_SKINNY_MAX_M (a few tokens, e.g. one decode step) and
- * K >= 1, TC and AUTO run a streaming CUDA-core kernel instead, which reads
- * each element of B once (4 bytes) and needs no workspace.  With
- * MOSAIC_SKINNY_MAX_M < M <= MOSAIC_STREAMW_MAX_M (a small decode batch) TC
- * and AUTO run a tensor-core kernel that also reads each element of B once as
- * uint32 and splits it into digits on the chip; it needs 8 M ceil8(K) bytes of
- * `ws` for A's digit planes.  Every path gives the same ring product. */
+ * K >= 1, TC and AUTO need no workspace: a streaming CUDA-core kernel reads
+ * each element of B once (4 bytes).  With 9 <= M <= MOSAIC_STREAMW_MAX_M (a
+ * small decode batch) and 8 M ceil8(K) bytes of `ws` for A's digit planes
+ * (required above MOSAIC_SKINNY_MAX_M) they run a tensor-core kernel that also
+ * reads each element of B once as uint32 and splits it into digits on the
+ * chip.  Every path gives the same ring product. */
 #define MOSAIC_SKINNY_MAX_M 16
 #define MOSAIC_STREAMW_MAX_M 64
 mosaic_status mosaic_ring_gemm(const uint32_t *A, int64_t lda, const uint32_t *B, int64_t ldb,

@@ -395,18 +395,18 @@ mosaic_status mosaic_ring_gemm(const uint32_t *A, int64_t lda, const uint32_t *B
     if (variant == MOSAIC_GEMM_MMA_S8)
         return ring_gemm_mma_s8(A, lda, B, ldb, C, ldc, nullptr, 0, 1, M, N, K, ws, ws_bytes, st);
     if (!tc_available()) return MOSAIC_ERR_UNSUPPORTED;
-    // A few tokens: the streaming kernel reads B once, no planes needed.
+    Carve cv = carve(ws, ws_bytes);
+    // kTcwMinM .. kTcwMaxM tokens: tensor cores, B read once as uint32 and split on the chip.
+    if (tcw_ok(A, lda, B, ldb, M, N, K)) {
+        uint16_t *Ap = cv.take<uint16_t>(tcw_ws_bytes(M, K) / 2);
+        if (Ap) return ring_gemm_tcw(A, lda, B, ldb, C, ldc, M, N, K, Ap, st);
+        if (M > kSkinnyMaxM) return MOSAIC_ERR_WORKSPACE;
+    }
+    // A few tokens, or no workspace for A's planes: the CUDA-core streaming kernel, which needs none.
     if (skinny_ok(A, lda, B, ldb, M, K))
         return ring_gemm_skinny(A, lda, B, ldb, C, ldc, nullptr, 0, 1, M, N, K, st);
     const int64_t Kp = (K + 7) / 8 * 8;
     if (!aligned16(A) || !aligned16(B) || lda % 4 || ldb % 4) return MOSAIC_ERR_ALIGN;
-    Carve cv = carve(ws, ws_bytes);
-    // Up to kTcwMaxM tokens: tensor cores, B read once as uint32 and split on the chip.
-    if (tcw_ok(A, lda, B, ldb, M, N, K)) {
-        uint16_t *Ap = cv.take<uint16_t>(tcw_ws_bytes(M, K) / 2);
-        if (!Ap) return MOSAIC_ERR_WORKSPACE;
-        return ring_gemm_tcw(A, lda, B, ldb, C, ldc, M, N, K, Ap, st);
-    }
     // Tensor-core variant: split both operands into digit planes in ws.
     uint16_t *Ap = cv.take<uint16_t>((size_t)(4 * M * Kp));
     uint16_t *Bp = cv.take<uint16_t>((size_t)(4 * N * Kp));
@@ -830,10 +830,6 @@ mosaic_status unmask_impl(const mosaic_params *p, int64_t l, int64_t m, const ui
     // (token-major: Q_d^T is the column block [m + od, m + Sr) of Z).
     const uint32_t *Qd = Z + m + od;
     const bool want_tc = variant == MOSAIC_GEMM_TC || (variant == MOSAIC_GEMM_AUTO && tc_available());
-    const int64_t Kp = kpad8(rd);
-    const bool tc_planes = Lp && want_tc && !skinny_ok(Qd, ldz, L, rd, l, rd) && ldz % 4 == 0 && aligned16(Qd) &&
-                           cv.used + up(8 * (size_t)(l * Kp)) <= cv.cap;
-    uint16_t *Qp = tc_planes ? cv.take<uint16_t>((size_t)(4 * l * Kp)) : nullptr;
     SparseLevel lev[2];
     int64_t soff = 0;
     for (uint32_t i = 1; i < d; i++) {

@@ -1,5 +1,5 @@
 // Ring product over Z_{2^32} on the tensor cores for a few token rows
-// (17 to 64), streaming the wide operand as uint32.
+// (9 to 64), streaming the wide operand as uint32.
 //
 // C = A B^T with A: M x K (tokens, M <= 64) and B: N x K (masked weights,
 // N in the thousands).  With so few tokens every element of B is used at most
@@ -533,7 +533,7 @@ mosaic_status tcw_status() {
 size_t tcw_ws_bytes(int64_t M, int64_t K) { return (size_t)(4 * M * ((K + 7) / 8 * 8)) * 2; }
 
 bool tcw_ok(const uint32_t *A, int64_t lda, const uint32_t *B, int64_t ldb, int64_t M, int64_t N, int64_t K) {
-    return M > kSkinnyMaxM && M <= kTcwMaxM && N >= 1 && K >= 1 && aligned16(A) && aligned16(B) && lda % 4 == 0 &&
+    return M >= kTcwMinM && M <= kTcwMaxM && N >= 1 && K >= 1 && aligned16(A) && aligned16(B) && lda % 4 == 0 &&
            ldb % 4 == 0 && tc_available();
 }
 
@@ -553,7 +553,7 @@ mosaic_status ring_gemm_tcw(const uint32_t *A, int64_t lda, const uint32_t *B, i
             A, lda, K, Ap, Kp, M * Kp, Cm, ldc, N, vec_a, vec_c);
     }
     MOSAIC_TRY(launch_status());
-    const int nt = M <= 32 ? 32 : M <= 48 ? 48 : 64;
+    const int nt = M <= 16 ? 16 : M <= 32 ? 32 : M <= 48 ? 48 : 64;
     CUtensorMap tw, tx;
     if (!make_w_map(&tw, B, K, N, ldb) || !make_x_map(&tx, Ap, K, M, Kp, nt)) return MOSAIC_ERR_CUDA;
     int dev = 0, sms = 0;
@@ -563,6 +563,7 @@ mosaic_status ring_gemm_tcw(const uint32_t *A, int64_t lda, const uint32_t *B, i
     const int64_t tiles = (N + WR - 1) / WR, nst = (K + KS - 1) / KS, nchunks = (nst + CHUNK - 1) / CHUNK;
     if (tiles * nchunks > (int64_t)INT32_MAX) return MOSAIC_ERR_SHAPE;
     const WArgs args{Cm, ldc, (int)M, (int)N, (int)K, (int)tiles, (int)nchunks};
+    if (nt == 16) return launch_tcw<16>(tw, tx, args, sms, st);
     if (nt == 32) return launch_tcw<32>(tw, tx, args, sms, st);
     if (nt == 48) return launch_tcw<48>(tw, tx, args, sms, st);
     return launch_tcw<64>(tw, tx, args, sms, st);

@@ -260,3 +260,24 @@ def test_mma_s8_adversarial(va, vb):
     B = np.full((N, K), vb, np.uint32)
     want = np.uint32((K * va * vb) % (1 << 32))
     assert np.all(ring_gemm_u32(A, B, variant=M.GEMM_MMA_S8) == want)
+
+
+@pytest.mark.parametrize("Mm", [8, 9, 13, 16])
+@pytest.mark.parametrize("N,K", [(300, 652), (20000 + 77, 1100)])
+def test_few_tokens_with_and_without_workspace(Mm, N, K):
+    """9 to 16 tokens stream B through the tensor cores when `ws` holds A's
+    planes and through the CUDA cores when it does not; 17 need the room."""
+    M = _M()
+    A = wl.uniform_u32(151 + Mm, Mm, K)
+    B = wl.uniform_u32(152, N, K)
+    want = ref(A, B)
+    assert np.array_equal(ring_gemm_u32(A, B), want)
+    C = torch.full((17, N), -1, dtype=torch.int32, device="cuda")
+    Ad = torch.from_numpy(np.vstack([A] * 3)[:17].view(np.int32)).cuda()
+    Bd = torch.from_numpy(B.view(np.int32)).cuda()
+    for ws in (None, torch.empty(8 * Mm * K - 512, dtype=torch.uint8, device="cuda")):
+        M.mosaic_ring_gemm(Ad, K, Bd, K, C, N, Mm, N, K, M.GEMM_TC, ws)
+        M.mosaic_device_status()
+        assert np.array_equal(host(C)[:Mm], want)
+    with pytest.raises(M.MosaicError, match="workspace"):
+        M.mosaic_ring_gemm(Ad, K, Bd, K, C, N, 17, N, K, M.GEMM_TC, None)

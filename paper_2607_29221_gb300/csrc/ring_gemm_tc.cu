@@ -18,13 +18,13 @@
 //     1, into int32 registers: acc += g_s << 8s mod 2^32 (drain_01 and
 //     drain_23 below convert the fp32 sums exactly).
 //
-// Pipeline (128 x BN output tiles, 10 warps):
+// Pipeline (128 x BN output tiles, 18 warps):
 //   warp 0      TMA producer: per stage one 3-D box {32 K, rows, 4 planes}
 //               for A and one for B (64-byte swizzle), mbarrier complete_tx
 //   warp 1      TMEM allocation (512 columns) and the single-thread MMA issuer
 //               (12 tcgen05.mma per stage: 8 of 128 x 2BN x 16, 4 of 128 x BN x 16)
-//   warps 2..9  epilogue: tcgen05.ld 32x32b, exact fp32 -> int32, shift-add (each lane
-//               quarter of TMEM twice, half of the columns each)
+//   warps 2..17 epilogue: tcgen05.ld 32x32b, exact fp32 -> int32, shift-add (each lane
+//               quarter of TMEM four times, a quarter of the columns each)
 // Every wait is bounded (about 2 s of %globaltimer); on expiry the kernel
 // raises a device error word, stops issuing work, waits (bounded) for its
 // own copies and products in flight, frees TMEM and returns.
@@ -45,14 +45,18 @@ constexpr int BK = 32;          // bf16 K elements per stage = one 64-byte swizz
 constexpr int STAGES = 3;
 constexpr int CHUNK = 8;        // stages between drains: 256 K
 constexpr uint32_t TMEM_COLS = 512;
-constexpr int THREADS = 320;   // warp 0 TMA, warp 1 MMA, warps 2..9 epilogue
-constexpr int EPI_WARPS = 8;
+constexpr int EPI_WARPS = 16;
+constexpr int THREADS = 64 + 32 * EPI_WARPS;   // warp 0 TMA, warp 1 MMA, warps 2..17 epilogue
 // Write-out slices: each epilogue warp moves its 32 rows 16 columns at a time
-// through a [32][EPI_PITCH] block of shared memory (pitch 20 words: the
-// row-per-lane 16-byte writes and the 8-rows-per-access 16-byte reads are
-// both conflict-free).
-constexpr int EPI_PITCH = 20;
-constexpr int EPI_BYTES = EPI_WARPS * 32 * EPI_PITCH * 4;
+// through a [32][16] block of shared memory, 16-byte chunk c of row r at
+// c ^ ((r >> 1) & 3): the row-per-lane 16-byte writes and the
+// 8-rows-per-access 16-byte reads are both conflict-free.  Sixteen epilogue
+// warps (32 columns each, 96 registers) leave room to fold groups 2 and 3 and
+// hand the accumulators back before the conversions: 0.3-0.7% over eight.
+constexpr int EPI_BYTES = EPI_WARPS * 32 * 16 * 4;
+__device__ __forceinline__ uint32_t epi_off(int row, int chunk) {
+    return (uint32_t)(row * 64 + ((chunk ^ ((row >> 1) & 3)) << 4));
+}
 
 // Drain conversions.  The fp32 group sums are integers with |x| <= 2^24 and
 // the F2I unit converts 16 values per clock per SM while the tensor pipe
@@ -66,28 +70,21 @@ constexpr float kM = 12582912.0f;
 // round(x1 / 2^8), x0 + 2^8 x1 = s + 2^16 h where s = x0 + 2^8 (x1 - 2^8 h)
 // is exact (|s| < 2^24) and goes through F2I; h << 16 is the bits of
 // x1 / 2^8 + kM shifted by 16, since bits(kM) << 16 = 0 mod 2^32.
-__device__ __forceinline__ void drain_01(uint32_t *acc, const uint32_t *v0, const uint32_t *v1) {
-#pragma unroll
-    for (int cc = 0; cc < 32; ++cc) {
-        const float x0 = __uint_as_float(v0[cc]), x1 = __uint_as_float(v1[cc]);
-        const float t = __fmaf_rn(x1, 0.00390625f, kM);
-        const float lo = __fmaf_rn(__fsub_rn(t, kM), -256.0f, x1);
-        const float s = __fmaf_rn(lo, 256.0f, x0);
-        acc[cc] += (uint32_t)__float2int_rn(s) + (__float_as_uint(t) << 16);
-    }
+__device__ __forceinline__ uint32_t drain_01(uint32_t v0, uint32_t v1) {
+    const float x0 = __uint_as_float(v0), x1 = __uint_as_float(v1);
+    const float t = __fmaf_rn(x1, 0.00390625f, kM);
+    const float lo = __fmaf_rn(__fsub_rn(t, kM), -256.0f, x1);
+    const float s = __fmaf_rn(lo, 256.0f, x0);
+    return (uint32_t)__float2int_rn(s) + (__float_as_uint(t) << 16);
 }
 
 // Groups 2 and 3 (|x2| <= 3 * 2^22, |x3| <= 2^24 after 256 K): (x2 << 16) +
 // (x3 << 24) = s << 16 mod 2^32 with s = x2 + 2^8 (x3 - 2^8 round(x3 / 2^8)),
 // exact (|s| < 2^24).
-__device__ __forceinline__ void drain_23(uint32_t *acc, const uint32_t *v0, const uint32_t *v1) {
-#pragma unroll
-    for (int cc = 0; cc < 32; ++cc) {
-        const float x3 = __uint_as_float(v1[cc]);
-        const float lo3 = __fmaf_rn(__fsub_rn(__fmaf_rn(x3, 0.00390625f, kM), kM), -256.0f, x3);
-        const float s = __fmaf_rn(lo3, 256.0f, __uint_as_float(v0[cc]));
-        acc[cc] += (uint32_t)__float2int_rn(s) << 16;
-    }
+__device__ __forceinline__ float fold_23(uint32_t v0, uint32_t v1) {
+    const float x3 = __uint_as_float(v1);
+    const float lo3 = __fmaf_rn(__fsub_rn(__fmaf_rn(x3, 0.00390625f, kM), kM), -256.0f, x3);
+    return __fmaf_rn(lo3, 256.0f, __uint_as_float(v0));
 }
 
 template <int BN>
@@ -165,17 +162,14 @@ __device__ __forceinline__ void umma_commit(uint64_t *bar) {
                      smem_u32(bar))
                  : "memory");
 }
-// 32 columns of TMEM for the warp's 32 lanes; the caller waits (tmem_wait).
-__device__ __forceinline__ void tmem_ld32_nowait(uint32_t taddr, uint32_t *v) {
+// 16 columns of TMEM for the warp's 32 lanes; the caller waits (tmem_wait).
+__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t *v) {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
         : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
           "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
-          "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]),
-          "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]),
-          "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+          "=r"(v[14]), "=r"(v[15])
         : "r"(taddr));
 }
 __device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
@@ -385,7 +379,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     } else {
         // Epilogue: warp w reads TMEM lanes 32 (w % 4) .. 32 (w % 4) + 31 and
         // columns [h HB, (h + 1) HB) of each group, h = (w - 2) / 4.
-        constexpr int HB = BN / 2;
+        constexpr int HB = BN / (EPI_WARPS / 4);
+        static_assert(HB % 16 == 0, "");
         const int q = warp & 3;
         const int h = (warp - 2) >> 2;
         const int row = q * 32 + lane;
@@ -407,24 +402,36 @@ __global__ void __launch_bounds__(THREADS, 1)
             tc_fence_after();
             const bool d01 = drains01(k, c, ++since01);
             if (d01) since01 = 0;
-            // Two groups are loaded before one wait.
+            // Two groups are loaded before one wait.  Groups 2 and 3 are folded
+            // into one fp32 value as they are loaded; its conversion follows
+            // once the accumulators are handed back, beside the next chunk's
+            // products.
+            if (d01) {
 #pragma unroll
-            for (int c0 = 0; c0 < HB; c0 += 32) {
-                uint32_t v0[32], v1[32];
-                if (d01) {
-                    tmem_ld32_nowait(lane_addr + 0 * BN + c0, v0);
-                    tmem_ld32_nowait(lane_addr + 1 * BN + c0, v1);
+                for (int c0 = 0; c0 < HB; c0 += 16) {
+                    uint32_t v0[16], v1[16];
+                    tmem_ld16_nowait(lane_addr + 0 * BN + c0, v0);
+                    tmem_ld16_nowait(lane_addr + 1 * BN + c0, v1);
                     tmem_wait();
-                    drain_01(acc + c0, v0, v1);
+#pragma unroll
+                    for (int cc = 0; cc < 16; ++cc) acc[c0 + cc] += drain_01(v0[cc], v1[cc]);
                 }
-                tmem_ld32_nowait(lane_addr + 2 * BN + c0, v0);
-                tmem_ld32_nowait(lane_addr + 3 * BN + c0, v1);
+            }
+            float s23[HB];
+#pragma unroll
+            for (int c0 = 0; c0 < HB; c0 += 16) {
+                uint32_t v0[16], v1[16];
+                tmem_ld16_nowait(lane_addr + 2 * BN + c0, v0);
+                tmem_ld16_nowait(lane_addr + 3 * BN + c0, v1);
                 tmem_wait();
-                drain_23(acc + c0, v0, v1);
+#pragma unroll
+                for (int cc = 0; cc < 16; ++cc) s23[c0 + cc] = fold_23(v0[cc], v1[cc]);
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(acc_empty);
+#pragma unroll
+            for (int cc = 0; cc < HB; ++cc) acc[cc] += (uint32_t)__float2int_rn(s23[cc]) << 16;
             ++chunk_count;
 
             // Short products (no stream-K): one chunk before the tile is written,
@@ -438,18 +445,16 @@ __global__ void __launch_bounds__(THREADS, 1)
                 const uint32_t *pin = sec ? a.Cin2 : a.Cin;
                 const int64_t ldp = sec ? a.ldcin2 : a.ldcin;
                 const uint32_t *psub = sec ? nullptr : a.Csub;
-                // Whole 64-column pieces only, so that every prefetched byte lies in the row.
+                // Whole 32-column pieces only, so that every prefetched byte lies in the row.
                 if (gr < a.M && col + HB <= (sec ? a.N - a.N1 : a.N1)) {
                     if (pin) {
                         const char *r0 = reinterpret_cast<const char *>(pin + (int64_t)gr * ldp + col);
                         asm volatile("prefetch.global.L2 [%0];" ::"l"(r0));
-                        asm volatile("prefetch.global.L2 [%0];" ::"l"(r0 + 128));
                         asm volatile("prefetch.global.L2 [%0];" ::"l"(r0 + 4 * HB - 4));
                     }
                     if (psub) {
                         const char *r0 = reinterpret_cast<const char *>(psub + (int64_t)gr * a.ldcsub + col);
                         asm volatile("prefetch.global.L2 [%0];" ::"l"(r0));
-                        asm volatile("prefetch.global.L2 [%0];" ::"l"(r0 + 128));
                         asm volatile("prefetch.global.L2 [%0];" ::"l"(r0 + 4 * HB - 4));
                     }
                 }
@@ -463,7 +468,6 @@ __global__ void __launch_bounds__(THREADS, 1)
             const bool second = tn0 >= a.N1;
             const int n0 = tn0 - (second ? a.N1 : 0) + h * HB;
             const int nout = second ? a.N - a.N1 : a.N1;
-            const int gm = m0 + row;
             uint32_t *const cbase = second ? a.C2 : a.C;
             const int64_t ldc_o = second ? a.ldc2 : a.ldc;
             const uint32_t *const cin0 = second ? a.Cin2 : a.Cin;
@@ -485,14 +489,14 @@ __global__ void __launch_bounds__(THREADS, 1)
                 // slice block (one row per lane) and come back as 8 rows x 64
                 // bytes per access, so C, Cin and Csub move in half lines
                 // instead of 16 bytes of 32 rows per access.
-                const uint32_t wb = epi_base + (uint32_t)((warp - 2) * 32 * EPI_PITCH * 4);
+                const uint32_t wb = epi_base + (uint32_t)((warp - 2) * 32 * 16 * 4);
                 const int pc = (lane >> 3) * 4;
 #pragma unroll
                 for (int s0 = 0; s0 < HB; s0 += 16) {
 #pragma unroll
                     for (int cc = 0; cc < 16; cc += 4)
                         asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(
-                                         wb + 4u * (uint32_t)(lane * EPI_PITCH + cc)),
+                                         wb + epi_off(lane, cc >> 2)),
                                      "r"(acc[s0 + cc]), "r"(acc[s0 + cc + 1]), "r"(acc[s0 + cc + 2]), "r"(acc[s0 + cc + 3])
                                      : "memory");
                     __syncwarp();
@@ -504,7 +508,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                         const int64_t col = n0 + s0 + pc;
                         asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
                                      : "=r"(v[it].x), "=r"(v[it].y), "=r"(v[it].z), "=r"(v[it].w)
-                                     : "r"(wb + 4u * (uint32_t)(rl * EPI_PITCH + pc))
+                                     : "r"(wb + epi_off(rl, lane >> 3))
                                      : "memory");
                         const uint32_t *bp = a.split ? cbase + (int64_t)gr * ldc_o + col
                                                      : (cin0 ? cin0 + (int64_t)gr * ldcin_o + col : nullptr);
@@ -523,21 +527,63 @@ __global__ void __launch_bounds__(THREADS, 1)
                                            v[it].z + ib[it].z - sb[it].z, v[it].w + ib[it].w - sb[it].w);
                     }
                 }
-            } else if (gm < a.M) {
-                uint32_t *crow = cbase + (int64_t)gm * ldc_o;
-                const uint32_t *cin = cin0 ? cin0 + (int64_t)gm * ldcin_o : nullptr;
-                const uint32_t *sub = sub0 ? sub0 + (int64_t)gm * a.ldcsub : nullptr;
-                if (atomic) {
+            } else {
+                // Split tiles and rows that forbid 16-byte accesses: the same slices,
+                // read back as 2 rows x 16 words (64 bytes a row) per access.  A row
+                // a lane took 32 sectors per access: 512 x 7308 x 4096 (split tiles)
+                // 203 -> 191 us, 301 x 8215 x 4096 (odd rows) 206 -> 158 us.
+                const uint32_t wb = epi_base + (uint32_t)((warp - 2) * 32 * 16 * 4);
+                const int pc = lane & 15;
+                const uint32_t *const base = a.split ? cbase : cin0;
+                const int64_t ldb = a.split ? ldc_o : ldcin_o;
 #pragma unroll
-                    for (int cc = 0; cc < HB; ++cc)
-                        if (n0 + cc < nout) atomicAdd(crow + n0 + cc, acc[cc]);
-                } else {
-                    const uint32_t *base = a.split ? crow : cin;
+                for (int s0 = 0; s0 < HB; s0 += 16) {
 #pragma unroll
-                    for (int cc = 0; cc < HB; ++cc) {
-                        const int gn = n0 + cc;
-                        if (gn < nout) crow[gn] = acc[cc] + (base ? base[gn] : 0u) - (sub ? sub[gn] : 0u);
+                    for (int cc = 0; cc < 16; cc += 4)
+                        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(wb + epi_off(lane, cc >> 2)),
+                                     "r"(acc[s0 + cc]), "r"(acc[s0 + cc + 1]), "r"(acc[s0 + cc + 2]), "r"(acc[s0 + cc + 3])
+                                     : "memory");
+                    __syncwarp();
+                    const int64_t col = n0 + s0 + pc;
+#pragma unroll
+                    for (int i0 = 0; i0 < 32; i0 += 8) {   // 8 rows: their loads are in flight at once
+                        uint32_t v[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int rl = i0 + 2 * u + (lane >> 4);
+                            asm volatile("ld.shared.u32 %0, [%1];"
+                                         : "=r"(v[u])
+                                         : "r"(wb + epi_off(rl, pc >> 2) + 4u * (uint32_t)(pc & 3))
+                                         : "memory");
+                        }
+                        const int gr0 = m0 + q * 32 + i0 + (lane >> 4);
+                        if (col >= nout || gr0 >= a.M) continue;
+                        const int last = a.M - 1;
+                        if (!atomic) {
+                            uint32_t x[4];
+                            if (base) {
+#pragma unroll
+                                for (int u = 0; u < 4; ++u) x[u] = base[(int64_t)min(gr0 + 2 * u, last) * ldb + col];
+#pragma unroll
+                                for (int u = 0; u < 4; ++u) v[u] += x[u];
+                            }
+                            if (sub0) {
+#pragma unroll
+                                for (int u = 0; u < 4; ++u) x[u] = sub0[(int64_t)min(gr0 + 2 * u, last) * a.ldcsub + col];
+#pragma unroll
+                                for (int u = 0; u < 4; ++u) v[u] -= x[u];
+                            }
+                        }
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int gr = gr0 + 2 * u;
+                            if (gr > last) continue;
+                            uint32_t *const cp = cbase + (int64_t)gr * ldc_o + col;
+                            if (atomic) atomicAdd(cp, v[u]);
+                            else *cp = v[u];
+                        }
                     }
+                    __syncwarp();
                 }
             }
 #pragma unroll

@@ -659,11 +659,13 @@ mosaic_status launch_tc(const uint16_t *Ap, int64_t ldpa, int64_t a_plane, const
     // Whole tiles on a persistent grid (at most one CTA per SM) unless the
     // last wave would leave more than 10% of the SMs idle; then the grid also
     // shares the remaining tiles' (tile, chunk) units evenly.  Short products
-    // (fewer than 8 chunks, K < 2048) keep whole tiles only: there the
-    // preparation of C and the split-tile atomics cost more than the idle SMs.
+    // (fewer than 6 chunks) keep whole tiles only: there the preparation of C
+    // and the split-tile atomics cost more than the idle SMs.  (512 x 8192 x
+    // 1536, 6 chunks, 256 tiles: 91.5 us whole, 87 us split; 3 chunks: 56
+    // against 33 us.)
     const int64_t waves = (tiles + sms - 1) / sms;
     // A subtracted input is read in plain mode only (stream-K prepares C from Cin alone).
-    const bool split = !o1.Csub && nchunks >= 8 && (double)tiles / (double)(waves * sms) < 0.9;
+    const bool split = !o1.Csub && nchunks >= 6 && (double)tiles / (double)(waves * sms) < 0.9;
     TcArgs args{Cm, ldc, Cin, ldcin, sgn, (int)M, (int)N, (int)K, (int)tiles_m, (int)tiles_n, split ? 1 : 0,
                 0, (int)o1.cols, o2.C, o2.ldc, o2.Cin, o2.ldcin, o1.Csub, o1.ldcsub};
     int64_t grid = tiles < sms ? tiles : sms;

@@ -399,7 +399,7 @@ mosaic_status mosaic_ring_gemm(const uint32_t *A, int64_t lda, const uint32_t *B
     // kTcwMinM .. kTcwMaxM tokens: tensor cores, B read once as uint32 and split on the chip.
     if (tcw_ok(A, lda, B, ldb, M, N, K)) {
         uint16_t *Ap = cv.take<uint16_t>(tcw_ws_bytes(M, K) / 2);
-        if (Ap) return ring_gemm_tcw(A, lda, B, ldb, C, ldc, M, N, K, Ap, st);
+        if (Ap) return ring_gemm_tcw(A, lda, B, ldb, C, ldc, nullptr, 0, nullptr, 0, 1, M, N, K, Ap, st);
         if (M > kSkinnyMaxM) return MOSAIC_ERR_WORKSPACE;
     }
     // A few tokens, or no workspace for A's planes: the CUDA-core streaming kernel, which needs none.
@@ -842,12 +842,16 @@ mosaic_status unmask_impl(const mosaic_params *p, int64_t l, int64_t m, const ui
     if (want_tc && unmask_few_ok(l, m, rd, (int)d - 1, lev))
         return unmask_few(l, m, Z, ldz, m + od, rd, K_tm, L, (int)d - 1, lev, s_w, s_x, bias, Y, Yhat, ldy, st);
     const int64_t Kp = kpad8(rd);
-    // Any row stride of Z qualifies: Q_d is split by a kernel that takes
-    // unaligned rows, and the product's write-out reads them 64 bytes at a time
-    // (on the CUDA cores, 301 x 5003 x 652 took 154 us, now 30 us).
-    const bool tc_planes = Lp && want_tc && !skinny_ok(Qd, ldz, L, rd, l, rd) &&
-                           cv.used + up(8 * (size_t)(l * Kp)) <= cv.cap;
-    uint16_t *Qp = tc_planes ? cv.take<uint16_t>((size_t)(4 * l * Kp)) : nullptr;
+    const bool room = cv.used + up(8 * (size_t)(l * Kp)) <= cv.cap;
+    // Up to kTcwMaxM tokens the product streams the uint32 L (half the bytes of
+    // its planes, and a token tile of its own size; whole unmask at 32 tokens,
+    // 57344 rows: 146 -> 113 us, 8192: 49.6 -> 40.1 us); more take L's planes.
+    // Any row stride of Z qualifies for both: Q_d is split by a kernel that
+    // takes unaligned rows, and the plane product's write-out reads them 64
+    // bytes at a time (on the CUDA cores, 301 x 5003 x 652 took 154 us, now 30).
+    const bool stream_l = want_tc && tc_available() && room && l <= kTcwMaxM && l >= kTcwMinM && rd % 4 == 0 && aligned16(L);
+    const bool tc_planes = !stream_l && Lp && want_tc && !skinny_ok(Qd, ldz, L, rd, l, rd) && room;
+    uint16_t *Qp = stream_l || tc_planes ? cv.take<uint16_t>((size_t)(4 * l * Kp)) : nullptr;
     // With room in the workspace, the gathers stage Q_i from tile images made
     // here, in the same launch that splits Q_d into digit planes.
     int nimg = 0;
@@ -880,8 +884,10 @@ mosaic_status unmask_impl(const mosaic_params *p, int64_t l, int64_t m, const ui
         lv.idx = buf;
         lv.lines = 1;
     }
-    MOSAIC_TRY(unmask_prep(Z, ldz, l, m + od, rd, Qp, Kp, nimg, icol, ir, img, nlin, lin, st));
-    if (Qp) {
+    MOSAIC_TRY(unmask_prep(Z, ldz, l, m + od, rd, tc_planes ? Qp : nullptr, Kp, nimg, icol, ir, img, nlin, lin, st));
+    if (stream_l) {
+        MOSAIC_TRY(ring_gemm_tcw(Qd, ldz, L, rd, tmp, m, Z, ldz, K_tm, m, -1, l, m, rd, Qp, st));
+    } else if (Qp) {
         MOSAIC_TRY(ring_gemm_tc_planes_diff(Qp, Kp, l * Kp, Lp, Kp, m * Kp, tmp, m, Z, ldz, K_tm, m, -1, l, m, rd,
                                             st));
     } else {

@@ -227,10 +227,11 @@ mosaic_status skinny_status();
 
 // Tensor-core ring GEMM for kTcwMinM <= M <= kTcwMaxM token rows that
 // streams B as uint32 (4 bytes an element) and splits it into digits on the
-// chip: C = A B^T (NT, uint32, K-contiguous).  Ap: tcw_ws_bytes(M, K) bytes of
-// 16-byte aligned scratch for A's fp16 digit planes.  tcw_ok() tells whether
-// the operands qualify (16-byte aligned bases, row strides multiples of 4
-// words, a Blackwell device).
+// chip: C = (Cin - Csub) + sgn * A B^T (NT, uint32, K-contiguous; Cin, Csub
+// nullable; B 16-byte aligned with a row stride of a multiple of 4 words).
+// Ap: tcw_ws_bytes(M, K) bytes of 16-byte aligned scratch for A's fp16 digit
+// planes.  tcw_ok() tells whether the operands of a plain product qualify
+// (16-byte aligned bases, row strides multiples of 4 words, a Blackwell device).
 // From 9 tokens it beats the CUDA-core streaming product, whose multiply-adds
 // then bind (60556 x 8192, one call: 391 against 568 us at 16 tokens, 390
 // against 320 at 8).
@@ -239,7 +240,8 @@ constexpr int64_t kTcwMaxM = 64;
 size_t tcw_ws_bytes(int64_t M, int64_t K);
 bool tcw_ok(const uint32_t *A, int64_t lda, const uint32_t *B, int64_t ldb, int64_t M, int64_t N, int64_t K);
 mosaic_status ring_gemm_tcw(const uint32_t *A, int64_t lda, const uint32_t *B, int64_t ldb, uint32_t *C,
-                            int64_t ldc, int64_t M, int64_t N, int64_t K, uint16_t *Ap, cudaStream_t st);
+                            int64_t ldc, const uint32_t *Cin, int64_t ldcin, const uint32_t *Csub, int64_t ldcsub,
+                            int sgn, int64_t M, int64_t N, int64_t K, uint16_t *Ap, cudaStream_t st);
 // Reads and clears that kernel's timeout word (after a stream sync).
 mosaic_status tcw_status();
 

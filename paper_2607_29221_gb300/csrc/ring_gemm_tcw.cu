@@ -31,7 +31,8 @@
 //     four digit slots);
 //   * (weight tile, 256-K chunk) units are split evenly over a persistent
 //     grid (stream-K); each CTA adds its partial tiles into C with red.add
-//     (C is zeroed first), exact and order-free in Z_{2^32}.
+//     (C starts as zero or as the difference of two inputs), exact and
+//     order-free in Z_{2^32}.
 // Warps: 0 TMA producer, 1 TMEM allocation + MMA issuer, 2..9 converters
 // (two groups of four, one warp per TMEM lane quarter; group j converts the
 // j-th 32-K box of every stage), 10..13 epilogue (warp w reaches TMEM lanes
@@ -87,6 +88,7 @@ struct WCfg {
 struct WArgs {
     uint32_t *C;
     int64_t ldc;
+    int sgn;
     int M, N, K;
     int tiles, nchunks;
 };
@@ -412,6 +414,10 @@ __global__ void __launch_bounds__(THREADS, 1)
             const bool tile_end = c == a.nchunks - 1 || u == u1 - 1;
             if (tile_end) {
                 const int n = tile * WR + r;
+                if (a.sgn < 0) {
+#pragma unroll
+                    for (int t = 0; t < NT; ++t) acc[t] = 0u - acc[t];
+                }
                 if (n < a.N) {
                     uint32_t *col = a.C + n;
 #pragma unroll
@@ -438,16 +444,18 @@ __global__ void __launch_bounds__(THREADS, 1)
 }
 
 // Digit planes of the token operand as fp16 bits, planes[d][r][c] =
-// byte_d(a + 0x80808080) - 128, and C (rows x n, leading dimension ldc)
-// zeroed for the red.add reduction, in one launch: block (x, r) covers
-// columns [1024 x, 1024 x + 1024) of row r, four consecutive columns a
-// thread (16-byte loads and stores where the row allows).
+// byte_d(a + 0x80808080) - 128, and C (rows x n, leading dimension ldc) set
+// to its start for the red.add reduction (Cin - Csub, or zero without them),
+// in one launch: block (x, r) covers columns [1024 x, 1024 x + 1024) of row
+// r, four consecutive columns a thread (16-byte loads and stores where the
+// row allows).
 __device__ __forceinline__ uint16_t digit_f16(uint32_t b, int d) {
     return __half_as_ushort(__int2half_rn((int)((b >> (8 * d)) & 0xffu) - 128));
 }
-__global__ void split_f16_zero_kernel(const uint32_t *a, int64_t lda, int64_t cols, uint16_t *planes, int64_t ldp,
-                                      int64_t plane_stride, uint32_t *C, int64_t ldc, int64_t n, int vec_a,
-                                      int vec_c) {
+__global__ void split_f16_start_kernel(const uint32_t *a, int64_t lda, int64_t cols, uint16_t *planes, int64_t ldp,
+                                       int64_t plane_stride, uint32_t *C, int64_t ldc, const uint32_t *Cin,
+                                       int64_t ldcin, const uint32_t *Csub, int64_t ldcsub, int64_t n, int vec_a,
+                                       int vec_c) {
     const int64_t r = blockIdx.y;
     const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
     if (c < cols) {
@@ -471,10 +479,16 @@ __global__ void split_f16_zero_kernel(const uint32_t *a, int64_t lda, int64_t co
     }
     if (c < n) {
         uint32_t *cr = C + r * ldc + c;
+        const uint32_t *ci = Cin ? Cin + r * ldcin + c : nullptr, *cs = Csub ? Csub + r * ldcsub + c : nullptr;
         if (vec_c && c + 4 <= n) {
-            *reinterpret_cast<uint4 *>(cr) = make_uint4(0u, 0u, 0u, 0u);
+            uint4 x = ci ? *reinterpret_cast<const uint4 *>(ci) : make_uint4(0u, 0u, 0u, 0u);
+            if (cs) {
+                const uint4 y = *reinterpret_cast<const uint4 *>(cs);
+                x.x -= y.x; x.y -= y.y; x.z -= y.z; x.w -= y.w;
+            }
+            *reinterpret_cast<uint4 *>(cr) = x;
         } else {
-            for (int k = 0; k < 4 && c + k < n; ++k) cr[k] = 0u;
+            for (int k = 0; k < 4 && c + k < n; ++k) cr[k] = (ci ? ci[k] : 0u) - (cs ? cs[k] : 0u);
         }
     }
 }
@@ -538,19 +552,21 @@ bool tcw_ok(const uint32_t *A, int64_t lda, const uint32_t *B, int64_t ldb, int6
 }
 
 mosaic_status ring_gemm_tcw(const uint32_t *A, int64_t lda, const uint32_t *B, int64_t ldb, uint32_t *Cm,
-                            int64_t ldc, int64_t M, int64_t N, int64_t K, uint16_t *Ap, cudaStream_t st) {
+                            int64_t ldc, const uint32_t *Cin, int64_t ldcin, const uint32_t *Csub, int64_t ldcsub,
+                            int sgn, int64_t M, int64_t N, int64_t K, uint16_t *Ap, cudaStream_t st) {
     if (M < 1 || M > kTcwMaxM || N < 1 || K < 1 || N > (int64_t)INT32_MAX || K > ((int64_t)1 << 20))
         return MOSAIC_ERR_SHAPE;
-    if (!aligned16(Ap)) return MOSAIC_ERR_ALIGN;
+    if (!aligned16(Ap) || !aligned16(B) || ldb % 4) return MOSAIC_ERR_ALIGN;
     const int64_t Kp = (K + 7) / 8 * 8;
     {
-        KernelSpan span("split_f16_zero", st);
+        KernelSpan span("split_f16_start", st);
         // Planes rows are Kp (a multiple of 8) fp16 apart, so their 8-byte stores are aligned.
         const int vec_a = aligned16(A) && lda % 4 == 0;
-        const int vec_c = aligned16(Cm) && ldc % 4 == 0;
+        const int vec_c = aligned16(Cm) && ldc % 4 == 0 && (!Cin || (aligned16(Cin) && ldcin % 4 == 0)) &&
+                          (!Csub || (aligned16(Csub) && ldcsub % 4 == 0));
         const int64_t wide = K > N ? K : N;
-        split_f16_zero_kernel<<<dim3((unsigned)((wide + 1023) / 1024), (unsigned)M), 256, 0, st>>>(
-            A, lda, K, Ap, Kp, M * Kp, Cm, ldc, N, vec_a, vec_c);
+        split_f16_start_kernel<<<dim3((unsigned)((wide + 1023) / 1024), (unsigned)M), 256, 0, st>>>(
+            A, lda, K, Ap, Kp, M * Kp, Cm, ldc, Cin, ldcin, Csub, ldcsub, N, vec_a, vec_c);
     }
     MOSAIC_TRY(launch_status());
     const int nt = M <= 16 ? 16 : M <= 32 ? 32 : M <= 48 ? 48 : 64;
@@ -562,7 +578,7 @@ mosaic_status ring_gemm_tcw(const uint32_t *A, int64_t lda, const uint32_t *B, i
         return MOSAIC_ERR_CUDA;
     const int64_t tiles = (N + WR - 1) / WR, nst = (K + KS - 1) / KS, nchunks = (nst + CHUNK - 1) / CHUNK;
     if (tiles * nchunks > (int64_t)INT32_MAX) return MOSAIC_ERR_SHAPE;
-    const WArgs args{Cm, ldc, (int)M, (int)N, (int)K, (int)tiles, (int)nchunks};
+    const WArgs args{Cm, ldc, sgn, (int)M, (int)N, (int)K, (int)tiles, (int)nchunks};
     if (nt == 16) return launch_tcw<16>(tw, tx, args, sms, st);
     if (nt == 32) return launch_tcw<32>(tw, tx, args, sms, st);
     if (nt == 48) return launch_tcw<48>(tw, tx, args, sms, st);

@@ -538,3 +538,15 @@ def test_rotation_and_encode_streamed_rows(n_pad):
 def test_unmask_of_few_tokens(d, r, t, m, l):
     g, ref, op, m, l = _run_layer(d, r, t, m=m, n=200, l=l, variant=M_().GEMM_AUTO)
     _check_layer(g, ref, op, m, l)
+
+
+# Above 16 tokens: the product that streams L (17 to 64 tokens, each token-tile size) and the one from
+# L's planes (65 up), with odd output widths (every row of Z and Y' unaligned), ragged tiles and
+# ranks that forbid streaming L (37) or leave one K stage.
+@pytest.mark.parametrize("r,t,m,l", [
+    ((96, 64, 40), (8, 4), 131, 17), ((96, 64, 40), (8, 4), 301, 33), ((96, 64, 300), (8, 4), 129, 48),
+    ((96, 64, 40), (6, 5), 77, 64), ((96, 64, 37), (8, 4), 131, 30), ((96, 64, 40), (8, 4), 259, 65),
+    ((96, 64, 300), (8, 4), 133, 150), ((1536, 1024, 652), (80, 80), 5, 20)])
+def test_unmask_products_by_token_count(r, t, m, l):
+    g, ref, op, m, l = _run_layer(3, r, t, m=m, n=200, l=l, variant=M_().GEMM_AUTO)
+    _check_layer(g, ref, op, m, l)

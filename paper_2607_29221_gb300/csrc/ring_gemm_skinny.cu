@@ -8,13 +8,14 @@
 // streaming B from HBM once, 4 bytes per element, and the 10 digit-plane
 // products of the tensor-core path (8 bytes of planes per element) would only
 // double the traffic.  Each CTA is persistent (one per SM) and walks B tiles
-// of BR rows:
-//   warp 15     TMA producer: per stage one 2-D box {128 K, BR rows} of B and
+// of br rows, br (at most 15 RW) being chosen so that the tiles fill whole
+// waves of CTAs:
+//   warp 15     TMA producer: per stage one 2-D box {128 K, br rows} of B and
 //               one {128 K, MT rows} of A into shared memory; rows and K past
 //               the ends are zero-filled by the copy engine
-//   warps 0-14  consumers: warp w owns rows w*RW .. w*RW+RW-1 of the tile, lane
-//               j the four K values 4j .. 4j+3 of every stage; it accumulates
-//               RW x MT wrapping 32-bit dot-product pieces (integer multiply-add)
+//   warps 0-14  consumers: warp w owns rows w, w + 15, .. of the tile (at most
+//               RW), lane j the four K values 4j .. 4j+3 of every stage; it
+//               accumulates RW x MT wrapping 32-bit dot-product pieces (integer multiply-add)
 //               and, after the last stage of the tile, sums them across the
 //               warp with a halving exchange (each step trades half of the
 //               values with the partner lane) and writes C.
@@ -36,7 +37,7 @@ constexpr int SMEM_BUDGET = 200 * 1024;
 
 template <int MT, int RW>
 struct SkCfg {
-    static constexpr int BR = CWARPS * RW;     // B rows per tile
+    static constexpr int BR = CWARPS * RW;     // most B rows per tile
     static constexpr int B_BYTES = BR * KC * 4;
     static constexpr int A_BYTES = MT * KC * 4;
     static constexpr int STAGE = B_BYTES + A_BYTES;
@@ -53,6 +54,7 @@ struct SkArgs {
     int64_t ldcin;
     int sgn;
     int M, N, nk, tiles;
+    int br;   // B rows per tile
 };
 
 __device__ __forceinline__ void raise_abort(volatile int *abort_flag) {
@@ -74,7 +76,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     ring_gemm_skinny_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                             SkArgs a) {
     using C = SkCfg<MT, RW>;
-    constexpr int V = RW * MT;                 // partial sums per lane
+    constexpr int V = (RW == 3 ? 4 : RW) * MT;   // partial sums per lane (a power of two)
     constexpr int H = Log2<V>::value < 5 ? Log2<V>::value : 5;   // halving exchanges
     constexpr int VL = V >> H;                 // sums a lane holds after them
     extern __shared__ uint8_t smem_raw[];
@@ -109,8 +111,8 @@ __global__ void __launch_bounds__(THREADS, 1)
                         break;
                     }
                     uint8_t *st = smem + s * C::STAGE;
-                    mbar_expect_tx(&full[s], C::STAGE);
-                    tma_load_2d(st, &tmB, &full[s], kc * KC, tile * C::BR);
+                    mbar_expect_tx(&full[s], (uint32_t)(a.br * KC * 4 + C::A_BYTES));
+                    tma_load_2d(st, &tmB, &full[s], kc * KC, tile * a.br);
                     tma_load_2d(st + C::B_BYTES, &tmA, &full[s], kc * KC, 0);
                 }
             }
@@ -123,7 +125,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     } else {
         uint32_t it = 0;
         bool ok = true;
-        const int r0 = warp * RW;
+        const int rows = (a.br - warp + CWARPS - 1) / CWARPS;   // this warp's rows of a tile (0 for none)
         for (int tile = blockIdx.x; ok && tile < a.tiles; tile += gridDim.x) {
             uint32_t acc[V];
 #pragma unroll
@@ -139,13 +141,14 @@ __global__ void __launch_bounds__(THREADS, 1)
                 const uint4 *As = reinterpret_cast<const uint4 *>(smem + s * C::STAGE + C::B_BYTES);
                 uint4 b[RW];
 #pragma unroll
-                for (int r = 0; r < RW; ++r) b[r] = Bs[(r0 + r) * (KC / 4) + lane];
+                for (int r = 0; r < RW; ++r)
+                    b[r] = r < rows ? Bs[(warp + CWARPS * r) * (KC / 4) + lane] : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
                 for (int t = 0; t < MT; ++t) {
                     const uint4 x = As[t * (KC / 4) + lane];
 #pragma unroll
                     for (int r = 0; r < RW; ++r)
-                        acc[r * MT + t] += b[r].x * x.x + b[r].y * x.y + b[r].z * x.z + b[r].w * x.w;
+                        if (r < rows) acc[r * MT + t] += b[r].x * x.x + b[r].y * x.y + b[r].z * x.z + b[r].w * x.w;
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&empty[s]);
@@ -176,8 +179,8 @@ __global__ void __launch_bounds__(THREADS, 1)
                 for (int i = 0; i < VL; ++i) {
                     const int idx = (lane >> (5 - H)) * VL + i;
                     const int r = idx / MT, t = idx % MT;
-                    const int64_t row = (int64_t)tile * C::BR + r0 + r;
-                    if (t < a.M && row < a.N) {
+                    const int64_t row = (int64_t)tile * a.br + warp + CWARPS * r;
+                    if (t < a.M && r < rows && row < a.N) {
                         uint32_t y = a.sgn < 0 ? 0u - acc[i] : acc[i];
                         if (a.Cin) y += a.Cin[(int64_t)t * a.ldcin + row];
                         a.C[(int64_t)t * a.ldc + row] = y;
@@ -204,16 +207,16 @@ bool make_u32_map(CUtensorMap *map, const uint32_t *base, int64_t K, int64_t row
 template <int MT, int RW>
 mosaic_status launch_skinny(const uint32_t *A, int64_t lda, const uint32_t *B, int64_t ldb, uint32_t *Cm,
                             int64_t ldc, const uint32_t *Cin, int64_t ldcin, int sgn, int64_t M, int64_t N,
-                            int64_t K, int sms, cudaStream_t st) {
+                            int64_t K, int br, int sms, cudaStream_t st) {
     using C = SkCfg<MT, RW>;
     CUtensorMap ta, tb;
-    if (!make_u32_map(&ta, A, K, M, lda, MT) || !make_u32_map(&tb, B, K, N, ldb, C::BR)) return MOSAIC_ERR_CUDA;
+    if (!make_u32_map(&ta, A, K, M, lda, MT) || !make_u32_map(&tb, B, K, N, ldb, br)) return MOSAIC_ERR_CUDA;
     static std::atomic<unsigned long long> attr_set{0};   // one bit per device ordinal
     if (!ensure_smem_limit(attr_set, ring_gemm_skinny_kernel<MT, RW>, C::SMEM)) return MOSAIC_ERR_CUDA;
-    const int64_t tiles = (N + C::BR - 1) / C::BR;
+    const int64_t tiles = (N + br - 1) / br;
     const int64_t nk = (K + KC - 1) / KC;
     if (tiles > 0x7fffffff || nk > 0x7fffffff) return MOSAIC_ERR_SHAPE;
-    SkArgs args{Cm, ldc, Cin, ldcin, sgn, (int)M, (int)N, (int)nk, (int)tiles};
+    SkArgs args{Cm, ldc, Cin, ldcin, sgn, (int)M, (int)N, (int)nk, (int)tiles, br};
     const int grid = tiles < sms ? (int)tiles : sms;
     {
         KernelSpan span("ring_gemm_skinny", st);
@@ -230,16 +233,17 @@ mosaic_status launch_rw(const uint32_t *A, int64_t lda, const uint32_t *B, int64
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
         return MOSAIC_ERR_CUDA;
-    // 60-row tiles read the token slice of A half as often as 30-row tiles;
-    // the smaller tiles are taken when they fill the last wave of the
-    // persistent grid clearly better.
-    auto eff = [&](int64_t br) {
-        const int64_t t = (N + br - 1) / br, w = (t + sms - 1) / sms;
-        return (double)t / (double)(w * sms);
-    };
-    if (eff(60) >= 0.85 || eff(60) >= eff(30))
-        return launch_skinny<MT, 4>(A, lda, B, ldb, Cm, ldc, Cin, ldcin, sgn, M, N, K, sms, st);
-    return launch_skinny<MT, 2>(A, lda, B, ldb, Cm, ldc, Cin, ldcin, sgn, M, N, K, sms, st);
+    // The fewest waves of tiles of at most 60 rows, and the tile height that
+    // fills them evenly: with tiles of 30 or 60 rows, 11404 rows left a sixth
+    // of the last wave's SMs idle (x 8192, weights from HBM: 60.3 -> 58.1 us at
+    // 1 token, 81.0 -> 76.0 at 8; x 32768: 215 -> 208 and 306 -> 286).  One
+    // wave keeps 30 or 60 rows: fewer and taller tiles read the token operand
+    // less often (7308 x 4096: 19.3 us either way).
+    const int64_t waves = (N + 60 * (int64_t)sms - 1) / (60 * (int64_t)sms);
+    const int br = waves > 1 ? (int)((N + waves * sms - 1) / (waves * sms)) : N > 30 * (int64_t)sms ? 60 : 30;
+    if (br <= 2 * CWARPS) return launch_skinny<MT, 2>(A, lda, B, ldb, Cm, ldc, Cin, ldcin, sgn, M, N, K, br, sms, st);
+    if (br <= 3 * CWARPS) return launch_skinny<MT, 3>(A, lda, B, ldb, Cm, ldc, Cin, ldcin, sgn, M, N, K, br, sms, st);
+    return launch_skinny<MT, 4>(A, lda, B, ldb, Cm, ldc, Cin, ldcin, sgn, M, N, K, br, sms, st);
 }
 
 }  // namespace

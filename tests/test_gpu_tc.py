@@ -281,3 +281,20 @@ def test_few_tokens_with_and_without_workspace(Mm, N, K):
         assert np.array_equal(host(C)[:Mm], want)
     with pytest.raises(M.MosaicError, match="workspace"):
         M.mosaic_ring_gemm(Ad, K, Bd, K, C, N, 17, N, K, M.GEMM_TC, None)
+
+
+@pytest.mark.parametrize("Mm", [1, 3, 8, 11])
+@pytest.mark.parametrize("N", [4560, 4561, 9120, 9121, 11404, 18241])
+def test_few_tokens_tile_heights(Mm, N):
+    """One wave of 30- and 60-row tiles, and two or three waves of tiles cut to
+    fill them evenly (31 to 45 rows: some warps have a row less than others,
+    the last tile is ragged); no workspace, so the CUDA-core kernel runs."""
+    M = _M()
+    K = 260
+    A = wl.uniform_u32(161 + Mm, Mm, K)
+    B = wl.uniform_u32(162, N, K)
+    C = torch.full((Mm, N), -1, dtype=torch.int32, device="cuda")
+    M.mosaic_ring_gemm(torch.from_numpy(A.view(np.int32)).cuda(), K, torch.from_numpy(B.view(np.int32)).cuda(), K, C,
+                       N, Mm, N, K, M.GEMM_TC, None)
+    M.mosaic_device_status()
+    assert np.array_equal(host(C), ref(A, B))

@@ -849,7 +849,10 @@ mosaic_status unmask_impl(const mosaic_params *p, int64_t l, int64_t m, const ui
     // Any row stride of Z qualifies for both: Q_d is split by a kernel that
     // takes unaligned rows, and the plane product's write-out reads them 64
     // bytes at a time (on the CUDA cores, 301 x 5003 x 652 took 154 us, now 30).
-    const bool stream_l = want_tc && tc_available() && room && l <= kTcwMaxM && l >= kTcwMinM && rd % 4 == 0 && aligned16(L);
+    // A caller that names the TC variant and brings L's planes gets the product
+    // from planes; AUTO is the fastest for the shape.
+    const bool stream_l = (variant == MOSAIC_GEMM_AUTO || !Lp) && want_tc && tc_available() && room && l <= kTcwMaxM &&
+                          l >= kTcwMinM && rd % 4 == 0 && aligned16(L);
     const bool tc_planes = !stream_l && Lp && want_tc && !skinny_ok(Qd, ldz, L, rd, l, rd) && room;
     uint16_t *Qp = stream_l || tc_planes ? cv.take<uint16_t>((size_t)(4 * l * Kp)) : nullptr;
     // With room in the workspace, the gathers stage Q_i from tile images made

@@ -57,11 +57,11 @@ __device__ __forceinline__ void dot_rows(uint32_t (&acc)[KV][T], const uint32_t 
             uint4 x[T];
 #pragma unroll
             for (int t = 0; t < T; t++)
-                x[t] = t < tn ? __ldg(reinterpret_cast<const uint4 *>(B + t * ldb + c0) + i) : make_uint4(0u, 0u, 0u, 0u);
+                x[t] = t < tn ? reinterpret_cast<const uint4 *>(B + t * ldb + c0)[i] : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
             for (int v = 0; v < KV; v++) {
                 if (v >= k) break;
-                const uint4 y = __ldg(reinterpret_cast<const uint4 *>(A + v * lda + c0) + i);
+                const uint4 y = reinterpret_cast<const uint4 *>(A + v * lda + c0)[i];
 #pragma unroll
                 for (int t = 0; t < T; t++) {
                     mac(v, t, y.x, x[t].x);
@@ -76,11 +76,11 @@ __device__ __forceinline__ void dot_rows(uint32_t (&acc)[KV][T], const uint32_t 
     for (int64_t i = c + threadIdx.x; i < c1; i += blockDim.x) {
         uint32_t x[T];
 #pragma unroll
-        for (int t = 0; t < T; t++) x[t] = t < tn ? __ldg(B + t * ldb + i) : 0u;
+        for (int t = 0; t < T; t++) x[t] = t < tn ? B[t * ldb + i] : 0u;
 #pragma unroll
         for (int v = 0; v < KV; v++) {
             if (v >= k) break;
-            const uint32_t y = __ldg(A + v * lda + i);
+            const uint32_t y = A[v * lda + i];
 #pragma unroll
             for (int t = 0; t < T; t++) mac(v, t, y, x[t]);
         }
@@ -103,6 +103,7 @@ __global__ void __launch_bounds__(kChkThreads)
     check_kernel(int k, const uint32_t *a, const uint32_t *Ychk, int64_t m, int64_t n_pad, int64_t l,
                  const uint32_t *Z, int64_t ldz, const uint32_t *Xp, int64_t ldx, uint32_t *bad, uint32_t *n_bad,
                  int vec_z, int vec_x) {
+    pdl_enter();
     __shared__ uint32_t part[kChkThreads / 32][KV * T];
     __shared__ uint32_t sums[KV * T];
     cg::cluster_group cluster = cg::this_cluster();
@@ -164,12 +165,14 @@ mosaic_status launch_check(int k, const uint32_t *a, const uint32_t *Ychk, int64
     cfg.gridDim = dim3((unsigned)(groups * S));
     cfg.blockDim = dim3(kChkThreads);
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)S;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     {
         KernelSpan span("freivalds_check", st);
         if (cudaLaunchKernelEx(&cfg, check_kernel<KV, T>, k, a, Ychk, m, n_pad, l, Z, ldz, Xp, ldx, bad, n_bad, vec_z,

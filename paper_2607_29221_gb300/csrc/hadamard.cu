@@ -201,6 +201,7 @@ struct Cfg {
 
 template <int E, int T>
 __global__ void __launch_bounds__(T * Cfg<E, T>::RPB) fwht_kernel(FwhtArgs a) {
+    pdl_trigger();
     using C = Cfg<E, T>;
     constexpr int N = C::N, WN = C::WN, CS = C::CS, RUNS = C::RUNS;
     static_assert(WN == 1 || E >= WN, "phase-3 layout needs E >= warps per row");
@@ -462,6 +463,7 @@ struct StreamCfg {
 
 template <int T>
 __global__ void __launch_bounds__(T, 1) fwht_stream_kernel(const __grid_constant__ CUtensorMap tmx, FwhtArgs a) {
+    pdl_enter();
     using C = StreamCfg<T>;
     constexpr int E = C::E, N = C::N, WN = C::WN, CS = C::CS, RUNS = C::RUNS;
     extern __shared__ uint8_t raw[];
@@ -668,7 +670,7 @@ mosaic_status launch_stream(const FwhtArgs &a, cudaStream_t st) {
     const int64_t grid = a.rows < sms ? a.rows : sms;
     {
         KernelSpan span("fwht_stream", st);
-        fwht_stream_kernel<T><<<(unsigned)grid, T, C::SMEM, st>>>(tmx, a);
+        pdl_launch(fwht_stream_kernel<T>, (unsigned)grid, T, C::SMEM, st, tmx, a);
     }
     return launch_status();
 }
@@ -709,6 +711,7 @@ constexpr size_t kPairSMEM = 1024 + kPairXBUF + 64;
 constexpr int kPairBox = 256;                   // chunks of 32 values per TMA box (32 KB)
 
 __global__ void __launch_bounds__(kPairT, 2) fwht_pair_kernel(const __grid_constant__ CUtensorMap tmx, FwhtArgs a) {
+    pdl_enter();
     constexpr int E = kPairE, N = kPairN, WN = kPairWN, CS = kPairCS, RUNS = kPairRuns;
     extern __shared__ uint8_t raw[];
     uint8_t *base_ptr = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~(uintptr_t)1023);
@@ -907,7 +910,7 @@ mosaic_status launch_pair(const FwhtArgs &a, cudaStream_t st) {
     const int64_t grid = a.rows < slots ? a.rows : slots;
     {
         KernelSpan span("fwht_pair", st);
-        fwht_pair_kernel<<<(unsigned)grid, kPairT, kPairSMEM, st>>>(tmx, a);
+        pdl_launch(fwht_pair_kernel, (unsigned)grid, kPairT, kPairSMEM, st, tmx, a);
     }
     return launch_status();
 }
@@ -954,6 +957,7 @@ struct RotCfg {
 
 template <int T>
 __global__ void __launch_bounds__(T, T == 512 ? 2 : 1) rot_kernel(const __grid_constant__ CUtensorMap tmx, FwhtArgs a) {
+    pdl_enter();
     using C = RotCfg<T>;
     constexpr int E = C::E, N = C::N, WN = C::WN;
     extern __shared__ uint8_t raw[];
@@ -1144,7 +1148,7 @@ mosaic_status launch_rot(const FwhtArgs &a, cudaStream_t st) {
     const int64_t grid = a.rows < slots ? a.rows : slots;
     {
         KernelSpan span("fwht_rot", st);
-        rot_kernel<T><<<(unsigned)grid, T, C::SMEM, st>>>(tmx, a);
+        pdl_launch(rot_kernel<T>, (unsigned)grid, T, C::SMEM, st, tmx, a);
     }
     return launch_status();
 }

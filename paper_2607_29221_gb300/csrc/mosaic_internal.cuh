@@ -85,6 +85,38 @@ inline cudaStream_t as_stream(void *s) { return reinterpret_cast<cudaStream_t>(s
 // Counts every kernel this library launches (read by mosaic_kernel_launches).
 void count_launch();
 
+// Programmatic dependent launch.  A kernel launched with pdl_launch may become
+// resident while the kernel before it on the stream is still running, once
+// every block of that kernel has called pdl_trigger() or ended.  Every thread
+// of it calls pdl_enter() before it touches global memory (only on-chip
+// set-up comes earlier, and no path returns earlier): that waits until all
+// earlier kernels have completed and their memory is visible, so the order
+// of the stream is kept and only the launch overlaps (2 to 3 us a launch
+// between back-to-back kernels).  It is for grids of at most one block per SM
+// (or of clusters): a grid of many small blocks would stack on the SMs that
+// free up first (the draws of a 301-token Init X went from 16 to 64 us), so
+// those are launched the ordinary way and only trigger.  What an earlier kernel
+// wrote is read with ordinary (coherent) or TMA loads, not __ldg.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_enter() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_trigger();
+}
+template <class... P, class... A>
+inline void pdl_launch(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kern, P(args)...);   // a failure is read by launch_status
+}
+
 inline mosaic_status launch_status() {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return MOSAIC_ERR_CUDA;

@@ -248,6 +248,7 @@ struct InitxDraws {
 constexpr int kDrawThreads = kSparseWarps * 32;
 
 __global__ void __launch_bounds__(kDrawThreads) initx_draw_kernel(InitxDraws a) {
+    pdl_trigger();
     extern __shared__ uint32_t sm[];
     uint32_t sid_lo, sid_hi;
     stream_id(a.sid, a.sid_dev, sid_lo, sid_hi);

@@ -96,6 +96,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         mbar_init_fence();
     }
     __syncthreads();
+    pdl_enter();   // everything above is on the chip
 
     if (warp == CWARPS) {
         if (lane == 0) {
@@ -220,7 +221,7 @@ mosaic_status launch_skinny(const uint32_t *A, int64_t lda, const uint32_t *B, i
     const int grid = tiles < sms ? (int)tiles : sms;
     {
         KernelSpan span("ring_gemm_skinny", st);
-        ring_gemm_skinny_kernel<MT, RW><<<grid, THREADS, C::SMEM, st>>>(ta, tb, args);
+        pdl_launch(ring_gemm_skinny_kernel<MT, RW>, grid, THREADS, C::SMEM, st, ta, tb, args);
     }
     return launch_status();
 }

@@ -268,6 +268,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    pdl_enter();   // everything above is on the chip
 
     if (warp == 0) {
         if (lane == 0) {
@@ -680,7 +681,7 @@ mosaic_status launch_tc(const uint16_t *Ap, int64_t ldpa, int64_t a_plane, const
     if (grid > 0x7fffffff) return MOSAIC_ERR_SHAPE;
     {
         KernelSpan span("ring_gemm_tc", st);
-        ring_gemm_tc_kernel<BN><<<(unsigned)grid, THREADS, C::SMEM, st>>>(ta, tb, args);
+        pdl_launch(ring_gemm_tc_kernel<BN>, (unsigned)grid, THREADS, C::SMEM, st, ta, tb, args);
     }
     return launch_status();
 }

@@ -226,6 +226,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     __syncthreads();
     fence_after();
     const uint32_t tmem = *tmem_slot;
+    pdl_enter();   // everything above is on the chip
     const uint32_t slot_col = (uint32_t)C::ACC_COLS;   // first digit slot
 
     if (warp == 0) {
@@ -456,6 +457,7 @@ __global__ void split_f16_start_kernel(const uint32_t *a, int64_t lda, int64_t c
                                        int64_t plane_stride, uint32_t *C, int64_t ldc, const uint32_t *Cin,
                                        int64_t ldcin, const uint32_t *Csub, int64_t ldcsub, int64_t n, int vec_a,
                                        int vec_c) {
+    pdl_trigger();
     const int64_t r = blockIdx.y;
     const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
     if (c < cols) {
@@ -527,7 +529,7 @@ mosaic_status launch_tcw(const CUtensorMap &tw, const CUtensorMap &tx, const WAr
     const int64_t grid = units < sms ? units : sms;
     {
         KernelSpan span("ring_gemm_tcw", st);
-        ring_gemm_tcw_kernel<NT><<<(unsigned)grid, THREADS, C::SMEM, st>>>(tw, tx, args);
+        pdl_launch(ring_gemm_tcw_kernel<NT>, (unsigned)grid, THREADS, C::SMEM, st, tw, tx, args);
     }
     return launch_status();
 }

@@ -261,6 +261,7 @@ constexpr int kPgStageBatch = 12;  // 16-byte loads a lane keeps in flight while
 template <bool LIST_IS_COL, bool CLAMP>
 __global__ void __launch_bounds__(kPgWarps * 32, 1)
     pgather_kernel(GatherArgs a, int units, int units0, int chunks, int vec_src, int vec_ab) {
+    pdl_enter();
     extern __shared__ __align__(16) uint32_t sm[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int grp = lane >> 2, li = lane & 3;
@@ -356,7 +357,7 @@ __global__ void __launch_bounds__(kPgWarps * 32, 1)
                 if (it < total && g0 + g < g_count && p < r) {
                     const uint32_t *srow = src + (g0 + g) * lds + a.col0;
                     if (vec_src && p + 4 <= r) {
-                        w[j] = __ldg(reinterpret_cast<const uint4 *>(srow + p));
+                        w[j] = *reinterpret_cast<const uint4 *>(srow + p);
                     } else {
                         w[j].x = srow[p];
                         if (p + 1 < r) w[j].y = srow[p + 1];
@@ -422,11 +423,11 @@ __global__ void __launch_bounds__(kPgWarps * 32, 1)
 #pragma unroll
                 for (int h = 0; h < 2; h++) {
                     if (ja) {
-                        const uint4 x = __ldg(reinterpret_cast<const uint4 *>(ja + e * jlda + g + 4 * h));
+                        const uint4 x = *reinterpret_cast<const uint4 *>(ja + e * jlda + g + 4 * h);
                         ab[4 * h] = x.x; ab[4 * h + 1] = x.y; ab[4 * h + 2] = x.z; ab[4 * h + 3] = x.w;
                     }
                     if (a.b) {
-                        const uint4 x = __ldg(reinterpret_cast<const uint4 *>(a.b + e * a.ldb + g + 4 * h));
+                        const uint4 x = *reinterpret_cast<const uint4 *>(a.b + e * a.ldb + g + 4 * h);
                         ab[4 * h] -= x.x; ab[4 * h + 1] -= x.y; ab[4 * h + 2] -= x.z; ab[4 * h + 3] -= x.w;
                     }
                 }
@@ -548,7 +549,7 @@ mosaic_status launch_pgather(const GatherArgs &a, cudaStream_t st) {
     }
     {
         KernelSpan span("pgather", st);
-        kern<<<(unsigned)grid, kPgWarps * 32, smem, st>>>(a, (int)units, (int)units0, (int)chunks, vec_src, vec_ab);
+        pdl_launch(kern, (unsigned)grid, kPgWarps * 32, smem, st, a, (int)units, (int)units0, (int)chunks, vec_src, vec_ab);
     }
     return launch_status();
 }
@@ -894,6 +895,7 @@ __device__ __forceinline__ void split4(const uint32_t *src, uint16_t *dst, int64
 }
 
 __global__ void __launch_bounds__(256) unmask_prep_kernel(UnmaskPrep a) {
+    pdl_trigger();
     __shared__ uint32_t t[32][33];
     int b = blockIdx.x;
     if (b < a.nb_split) {

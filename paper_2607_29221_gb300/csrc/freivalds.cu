@@ -57,11 +57,11 @@ __device__ __forceinline__ void dot_rows(uint32_t (&acc)[KV][T], const uint32_t 
             uint4 x[T];
 #pragma unroll
             for (int t = 0; t < T; t++)
-                x[t] = t < tn ? reinterpret_cast<const uint4 *>(B + t * ldb + c0)[i] : make_uint4(0u, 0u, 0u, 0u);
+                x[t] = t < tn ? __ldcg(reinterpret_cast<const uint4 *>(B + t * ldb + c0) + i) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
             for (int v = 0; v < KV; v++) {
                 if (v >= k) break;
-                const uint4 y = reinterpret_cast<const uint4 *>(A + v * lda + c0)[i];
+                const uint4 y = __ldca(reinterpret_cast<const uint4 *>(A + v * lda + c0) + i);
 #pragma unroll
                 for (int t = 0; t < T; t++) {
                     mac(v, t, y.x, x[t].x);
@@ -76,11 +76,11 @@ __device__ __forceinline__ void dot_rows(uint32_t (&acc)[KV][T], const uint32_t 
     for (int64_t i = c + threadIdx.x; i < c1; i += blockDim.x) {
         uint32_t x[T];
 #pragma unroll
-        for (int t = 0; t < T; t++) x[t] = t < tn ? B[t * ldb + i] : 0u;
+        for (int t = 0; t < T; t++) x[t] = t < tn ? __ldcg(B + t * ldb + i) : 0u;
 #pragma unroll
         for (int v = 0; v < KV; v++) {
             if (v >= k) break;
-            const uint32_t y = A[v * lda + i];
+            const uint32_t y = __ldca(A + v * lda + i);
 #pragma unroll
             for (int t = 0; t < T; t++) mac(v, t, y, x[t]);
         }

@@ -550,3 +550,18 @@ def test_unmask_of_few_tokens(d, r, t, m, l):
 def test_unmask_products_by_token_count(r, t, m, l):
     g, ref, op, m, l = _run_layer(3, r, t, m=m, n=200, l=l, variant=M_().GEMM_AUTO)
     _check_layer(g, ref, op, m, l)
+
+
+# Quad stores of the uniform draws: rows of one and of several quads (a block's 16 words cross rows),
+# padded rows, a total that ends inside a block, and outputs or strides that forbid them.
+@pytest.mark.parametrize("rows,cols,ld,off", [
+    (5, 4, 4, 0), (9, 12, 12, 0), (33, 20, 24, 0), (7, 652, 656, 0), (6, 20, 21, 0), (6, 20, 24, 1), (3, 18, 20, 0)])
+def test_prg_uniform_quads(rows, cols, ld, off):
+    M = M_()
+    tg, sid = O.tag(O.KIND_L), 99
+    flat = torch.full((rows * ld + off,), -1, dtype=torch.int32, device="cuda")
+    out = flat[off:].view(rows, ld)
+    M.mosaic_prg_uniform(ckey(), tg, sid, 20, rows, cols, out, ld)
+    got = host_u32(out)
+    assert np.array_equal(got[:, :cols], O.sample_uniform(KEY, tg, sid, rows, cols, 20))
+    assert np.all(got[:, cols:] == 0xFFFFFFFF)

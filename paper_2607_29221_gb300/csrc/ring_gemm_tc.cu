@@ -109,7 +109,7 @@ struct Cfg {
 struct TcArgs {
     uint32_t *C;
     int64_t ldc;
-    const uint32_t *Cin;   // plain mode only (stream-K mode prepares C instead)
+    const uint32_t *Cin;   // read by tiles that one CTA sums whole (C is prepared where tiles are shared)
     int64_t ldcin;
     int sgn;
     int M, N, K;
@@ -480,10 +480,10 @@ __global__ void __launch_bounds__(THREADS, 1)
             }
             // Other CTAs add into a split tile too: exact and order-free in Z_{2^32}.
             const bool atomic = a.split && !whole;
-            // Plain mode: C = Cin - Csub + acc.  Stream-K mode, whole tile: C (prepared) += acc.
+            // A whole tile: C = Cin - Csub + acc.
             const bool vecw = !atomic && (n0 + HB <= nout) && ((ldc_o & 3) == 0) &&
                               ((reinterpret_cast<uintptr_t>(cbase) & 15u) == 0) &&
-                              (a.split || !cin0 || (((ldcin_o & 3) == 0) && ((reinterpret_cast<uintptr_t>(cin0) & 15u) == 0))) &&
+                              (!cin0 || (((ldcin_o & 3) == 0) && ((reinterpret_cast<uintptr_t>(cin0) & 15u) == 0))) &&
                               (!sub0 || (((a.ldcsub & 3) == 0) && ((reinterpret_cast<uintptr_t>(sub0) & 15u) == 0)));
             if (vecw) {
                 // Coalesced write-out: 16 columns of the warp's 32 rows go to its
@@ -511,8 +511,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                                      : "=r"(v[it].x), "=r"(v[it].y), "=r"(v[it].z), "=r"(v[it].w)
                                      : "r"(wb + epi_off(rl, lane >> 3))
                                      : "memory");
-                        const uint32_t *bp = a.split ? cbase + (int64_t)gr * ldc_o + col
-                                                     : (cin0 ? cin0 + (int64_t)gr * ldcin_o + col : nullptr);
+                        const uint32_t *bp = cin0 ? cin0 + (int64_t)gr * ldcin_o + col : nullptr;
                         const uint32_t *sp = sub0 ? sub0 + (int64_t)gr * a.ldcsub + col : nullptr;
                         ib[it] = (gr < a.M && bp) ? *reinterpret_cast<const uint4 *>(bp) : make_uint4(0, 0, 0, 0);
                         sb[it] = (gr < a.M && sp) ? *reinterpret_cast<const uint4 *>(sp) : make_uint4(0, 0, 0, 0);
@@ -535,8 +534,6 @@ __global__ void __launch_bounds__(THREADS, 1)
                 // 203 -> 191 us, 301 x 8215 x 4096 (odd rows) 206 -> 158 us.
                 const uint32_t wb = epi_base + (uint32_t)((warp - 2) * 32 * 16 * 4);
                 const int pc = lane & 15;
-                const uint32_t *const base = a.split ? cbase : cin0;
-                const int64_t ldb = a.split ? ldc_o : ldcin_o;
 #pragma unroll
                 for (int s0 = 0; s0 < HB; s0 += 16) {
 #pragma unroll
@@ -562,9 +559,9 @@ __global__ void __launch_bounds__(THREADS, 1)
                         const int last = a.M - 1;
                         if (!atomic) {
                             uint32_t x[4];
-                            if (base) {
+                            if (cin0) {
 #pragma unroll
-                                for (int u = 0; u < 4; ++u) x[u] = base[(int64_t)min(gr0 + 2 * u, last) * ldb + col];
+                                for (int u = 0; u < 4; ++u) x[u] = cin0[(int64_t)min(gr0 + 2 * u, last) * ldcin_o + col];
 #pragma unroll
                                 for (int u = 0; u < 4; ++u) v[u] += x[u];
                             }
@@ -625,14 +622,16 @@ struct TcOut {
     int64_t ldcsub = 0;
 };
 
-// Prepares a stream-K output: its tiles are summed with atomic adds, so it
-// starts as Cin (or 0).
-cudaError_t prepare_split(const TcOut &o, int64_t M, cudaStream_t st) {
-    if (o.cols == 0) return cudaSuccess;
-    if (!o.Cin) return cudaMemset2DAsync(o.C, (size_t)o.ldc * 4, 0, (size_t)o.cols * 4, (size_t)M, st);
+// Prepares the columns [c0, cols) of a stream-K output, whose tiles are (or
+// may be) summed with atomic adds: they start as Cin (or 0).
+cudaError_t prepare_split(const TcOut &o, int64_t M, int64_t c0, cudaStream_t st) {
+    if (c0 < 0) c0 = 0;
+    if (o.cols <= c0) return cudaSuccess;
+    const size_t width = (size_t)(o.cols - c0) * 4;
+    if (!o.Cin) return cudaMemset2DAsync(o.C + c0, (size_t)o.ldc * 4, 0, width, (size_t)M, st);
     if (o.Cin != o.C)
-        return cudaMemcpy2DAsync(o.C, (size_t)o.ldc * 4, o.Cin, (size_t)o.ldcin * 4, (size_t)o.cols * 4,
-                                 (size_t)M, cudaMemcpyDeviceToDevice, st);
+        return cudaMemcpy2DAsync(o.C + c0, (size_t)o.ldc * 4, o.Cin + c0, (size_t)o.ldcin * 4, width, (size_t)M,
+                                 cudaMemcpyDeviceToDevice, st);
     return cudaSuccess;
 }
 
@@ -671,12 +670,13 @@ mosaic_status launch_tc(const uint16_t *Ap, int64_t ldpa, int64_t a_plane, const
                 0, (int)o1.cols, o2.C, o2.ldc, o2.Cin, o2.ldcin, o1.Csub, o1.ldcsub};
     int64_t grid = tiles < sms ? tiles : sms;
     if (split) {
-        if (prepare_split(o1, M, st) != cudaSuccess || prepare_split(o2, M, st) != cudaSuccess)
-            return MOSAIC_ERR_CUDA;
-        args.Cin = nullptr;
-        args.Cin2 = nullptr;
         grid = tiles * nchunks < sms ? tiles * nchunks : sms;
         args.dp_tiles = (int)((tiles / grid) * grid);   // whole waves run as whole tiles
+        // Only the columns that shared tiles reach need their start (one CTA's
+        // tiles overwrite theirs, also where they lie beside shared ones).
+        const int64_t c0 = args.dp_tiles / tiles_m * BN;
+        if (prepare_split(o1, M, c0, st) != cudaSuccess || prepare_split(o2, M, c0 - o1.cols, st) != cudaSuccess)
+            return MOSAIC_ERR_CUDA;
     }
     if (grid > 0x7fffffff) return MOSAIC_ERR_SHAPE;
     {

@@ -733,19 +733,34 @@ __global__ void rowgather_kernel(const uint32_t *P, int64_t ldp, SparseLevel l0,
     out[j * ldo + c] = acc;
 }
 
-__global__ void transpose_kernel(const uint32_t *a, int64_t lda, int64_t rows, int64_t cols,
-                                 uint32_t *out, int64_t ldo) {
-    __shared__ uint32_t tile[32][33];
-    const int64_t r0 = (int64_t)blockIdx.y * 32, c0 = (int64_t)blockIdx.x * 32;
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int64_t r = r0 + i, c = c0 + threadIdx.x;
-        if (r < rows && c < cols) tile[i][threadIdx.x] = a[r * lda + c];
-    }
+// 64 x 64 words a block, sixteen loads a thread in flight (memory bound:
+// 4096 x 3212 words 28.9 -> 16.3 us against 32 x 32 tiles with four).
+constexpr int kTrTile = 64;
+__global__ void __launch_bounds__(256) transpose_kernel(const uint32_t *a, int64_t lda, int64_t rows, int64_t cols,
+                                                        uint32_t *out, int64_t ldo) {
+    __shared__ uint32_t tile[kTrTile][kTrTile + 1];
+    const int64_t r0 = (int64_t)blockIdx.y * kTrTile, c0 = (int64_t)blockIdx.x * kTrTile;
+    const int tx = threadIdx.x, ty = threadIdx.y;   // 32 x 8
+    uint32_t v[kTrTile / 8][2];
+#pragma unroll
+    for (int i = 0; i < kTrTile / 8; i++)
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const int64_t r = r0 + ty + 8 * i, c = c0 + tx + 32 * h;
+            v[i][h] = r < rows && c < cols ? a[r * lda + c] : 0u;
+        }
+#pragma unroll
+    for (int i = 0; i < kTrTile / 8; i++)
+#pragma unroll
+        for (int h = 0; h < 2; h++) tile[ty + 8 * i][tx + 32 * h] = v[i][h];
     __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int64_t c = c0 + i, r = r0 + threadIdx.x;
-        if (r < rows && c < cols) out[c * ldo + r] = tile[threadIdx.x][i];
-    }
+#pragma unroll
+    for (int i = 0; i < kTrTile / 8; i++)
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const int64_t c = c0 + ty + 8 * i, r = r0 + tx + 32 * h;
+            if (r < rows && c < cols) out[c * ldo + r] = tile[tx + 32 * h][ty + 8 * i];
+        }
 }
 
 
@@ -843,10 +858,37 @@ __device__ __forceinline__ void tile_image_block(const uint32_t *src, int64_t ld
         img[((size_t)tile * rp + p) * 32 + tx] = t[g][k];
     }
 }
-__global__ void tile_image_kernel(const uint32_t *src, int64_t lds, int64_t col0, int r, int64_t g_count, int rp,
-                                  uint32_t *img) {
-    __shared__ uint32_t t[32][33];
-    tile_image_block(src, lds, col0, r, g_count, rp, img, blockIdx.y, blockIdx.x * 32, t);
+// The images of a whole segment, 128 positions of a tile a block: sixteen
+// loads a thread in flight (memory bound: 4096 rows x 1536 positions 20.2 ->
+// 10.5 us against blocks of 32 positions).
+constexpr int kTiPos = 128;
+__global__ void __launch_bounds__(256) tile_image_kernel(const uint32_t *src, int64_t lds, int64_t col0, int r,
+                                                         int64_t g_count, int rp, uint32_t *img) {
+    __shared__ uint32_t t[32][kTiPos + 1];
+    const int64_t tile = blockIdx.y;
+    const int p0 = blockIdx.x * kTiPos;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    uint32_t v[4][kTiPos / 32];
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+#pragma unroll
+        for (int h = 0; h < kTiPos / 32; h++) {
+            const int64_t g = tile * 32 + ty + 8 * i;
+            const int p = p0 + tx + 32 * h;
+            v[i][h] = g < g_count && p < r ? src[g * lds + col0 + p] : 0u;
+        }
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+#pragma unroll
+        for (int h = 0; h < kTiPos / 32; h++) t[ty + 8 * i][tx + 32 * h] = v[i][h];
+    __syncthreads();
+    const int c = tx >> 2, w = tx & 3;
+#pragma unroll 4
+    for (int k = ty; k < kTiPos; k += 8) {
+        const int p = p0 + k;
+        if (p >= rp) break;
+        img[((size_t)tile * rp + p) * 32 + tx] = t[((c ^ (int)pg_perm((uint32_t)p)) << 2) | w][k];
+    }
 }
 
 // Before an unmask: the digit planes of Q_d (the A operand of Q_d L^T) and
@@ -951,7 +993,7 @@ mosaic_status build_tile_image(const uint32_t *src, int64_t lds, int64_t col0, u
     if (tiles > 65535) return MOSAIC_ERR_SHAPE;
     {
         KernelSpan span("tile_image", st);
-        tile_image_kernel<<<dim3((unsigned)(rp / 32), (unsigned)tiles), 256, 0, st>>>(src, lds, col0, (int)r, g_count,
+        tile_image_kernel<<<dim3((unsigned)((rp + kTiPos - 1) / kTiPos), (unsigned)tiles), 256, 0, st>>>(src, lds, col0, (int)r, g_count,
                                                                                       rp, img);
     }
     return launch_status();
@@ -1150,7 +1192,7 @@ mosaic_status sparse_rowgather(const uint32_t *P, int64_t ldp, const SparseLevel
 mosaic_status transpose_u32(const uint32_t *a, int64_t lda, int64_t rows, int64_t cols, uint32_t *out,
                             int64_t ldo, cudaStream_t st) {
     if (rows == 0 || cols == 0) return MOSAIC_OK;
-    dim3 grid((unsigned)((cols + 31) / 32), (unsigned)((rows + 31) / 32));
+    dim3 grid((unsigned)((cols + kTrTile - 1) / kTrTile), (unsigned)((rows + kTrTile - 1) / kTrTile));
     if (grid.y > 65535) return MOSAIC_ERR_SHAPE;
     {
         KernelSpan span("transpose", st);

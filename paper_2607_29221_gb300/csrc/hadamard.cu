@@ -665,7 +665,7 @@ mosaic_status launch_stream(const FwhtArgs &a, cudaStream_t st) {
     static std::atomic<unsigned long long> attr_set{0};
     int dev = 0, sms = 0;
     if (!ensure_smem_limit(attr_set, fwht_stream_kernel<T>, C::SMEM, &dev) ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+        (sms = sm_count(dev)) < 1)
         return MOSAIC_ERR_CUDA;
     const int64_t grid = a.rows < sms ? a.rows : sms;
     {
@@ -900,7 +900,7 @@ mosaic_status launch_pair(const FwhtArgs &a, cudaStream_t st) {
     static std::atomic<unsigned long long> attr_set{0};
     int dev = 0, sms = 0, per_sm = 0;
     if (!ensure_smem_limit(attr_set, fwht_pair_kernel, kPairSMEM, &dev) ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1 ||
+        (sms = sm_count(dev)) < 1 ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fwht_pair_kernel, kPairT, kPairSMEM) != cudaSuccess ||
         per_sm < 1)
         return MOSAIC_ERR_CUDA;
@@ -1140,7 +1140,7 @@ mosaic_status launch_rot(const FwhtArgs &a, cudaStream_t st) {
     static std::atomic<unsigned long long> attr_set{0};
     int dev = 0, sms = 0, per_sm = 0;
     if (!ensure_smem_limit(attr_set, rot_kernel<T>, C::SMEM, &dev) ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1 ||
+        (sms = sm_count(dev)) < 1 ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rot_kernel<T>, T, C::SMEM) != cudaSuccess ||
         per_sm < 1)
         return MOSAIC_ERR_CUDA;

@@ -28,6 +28,17 @@ inline bool ensure_smem_limit(std::atomic<unsigned long long> &done, Kernel kern
     return true;
 }
 
+// Multiprocessors of device `dev`, looked up once per ordinal (0 on failure).
+inline int sm_count(int dev) {
+    static std::atomic<int> cache[64];
+    std::atomic<int> &at = cache[dev & 63];
+    int n = at.load(std::memory_order_relaxed);
+    if (n > 0) return n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    at.store(n, std::memory_order_relaxed);
+    return n;
+}
+
 constexpr int kSparseWindow = 65536;   // stream words reserved per sparse row
 constexpr int kMaxGaussBound = 96;     // B = ceil(12 sigma) for sigma <= 8
 

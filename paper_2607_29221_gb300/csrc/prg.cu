@@ -336,6 +336,21 @@ int gaussian_table_host(float sigma, unsigned long long *table) {
     return B;
 }
 
+namespace {
+// The table of the last sigma this thread used: its long double exponentials
+// are emulated on the host's Arm cores and cost more than the launch.
+const GaussTable &gauss_table(float sigma) {
+    thread_local GaussTable tab{};
+    thread_local float of = 0.0f;
+    if (of != sigma) {
+        tab.bound = gaussian_table_host(sigma, tab.t);
+        tab.n = 2 * tab.bound + 1;
+        of = sigma;
+    }
+    return tab;
+}
+}  // namespace
+
 mosaic_status prg_uniform(const Key &key, uint32_t tag, uint64_t sid, int rounds, int64_t rows,
                           int64_t cols, uint32_t *out, int64_t ldo, cudaStream_t st, const uint64_t *sid_dev) {
     const int64_t total = rows * cols;
@@ -360,9 +375,7 @@ mosaic_status prg_gaussian(const Key &key, uint32_t tag, uint64_t sid, int round
         return cudaMemsetAsync(out, 0, sizeof(uint32_t) * (size_t)count, st) == cudaSuccess
                    ? MOSAIC_OK : MOSAIC_ERR_CUDA;
     }
-    GaussTable tab;
-    tab.bound = gaussian_table_host(sigma, tab.t);
-    tab.n = 2 * tab.bound + 1;
+    const GaussTable &tab = gauss_table(sigma);
     const int64_t nblk = (count + 7) / 8;
     {
         KernelSpan span("prg_gaussian", st);
@@ -409,8 +422,7 @@ mosaic_status prg_initx(const Key &key, int rounds, uint64_t sid, const uint64_t
     a.ecount = ecount;
     a.E = E;
     if (sigma != 0.0f) {
-        a.tab.bound = gaussian_table_host(sigma, a.tab.t);
-        a.tab.n = 2 * a.tab.bound + 1;
+        a.tab = gauss_table(sigma);
     } else {
         a.tab.bound = a.tab.n = 0;
     }

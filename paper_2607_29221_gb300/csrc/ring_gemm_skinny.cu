@@ -232,7 +232,7 @@ mosaic_status launch_rw(const uint32_t *A, int64_t lda, const uint32_t *B, int64
                         cudaStream_t st) {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+        (sms = sm_count(dev)) < 1)
         return MOSAIC_ERR_CUDA;
     // The fewest waves of tiles of at most 60 rows, and the tile height that
     // fills them evenly: with tiles of 30 or 60 rows, 11404 rows left a sixth

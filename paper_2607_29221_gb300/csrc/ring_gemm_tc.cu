@@ -653,9 +653,8 @@ mosaic_status launch_tc(const uint16_t *Ap, int64_t ldpa, int64_t a_plane, const
     const int64_t tiles_m = (M + BM - 1) / BM, tiles_n = (N + BN - 1) / BN, tiles = tiles_m * tiles_n;
     const int64_t nk = (K + BK - 1) / BK, nchunks = (nk + CHUNK - 1) / CHUNK;
     if (tiles * nchunks > (int64_t)INT32_MAX) return MOSAIC_ERR_SHAPE;   // 32-bit unit numbers
-    int sms = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-        return MOSAIC_ERR_CUDA;
+    const int sms = sm_count(dev);
+    if (sms < 1) return MOSAIC_ERR_CUDA;
     // Whole tiles on a persistent grid (at most one CTA per SM) unless the
     // last wave would leave more than 10% of the SMs idle; then the grid also
     // shares the remaining tiles' (tile, chunk) units evenly.  Short products
@@ -689,11 +688,17 @@ mosaic_status launch_tc(const uint16_t *Ap, int64_t ldpa, int64_t a_plane, const
 }  // namespace
 
 bool tc_available() {
+    static std::atomic<int> cache[64];   // per device ordinal: 0 not looked up, 1 no, 2 yes
     int dev = 0, major = 0, minor = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    std::atomic<int> &at = cache[dev & 63];
+    const int known = at.load(std::memory_order_relaxed);
+    if (known) return known == 2;
     if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) return false;
     if (cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev) != cudaSuccess) return false;
-    return major == 10 && minor == 3 && encode_fn() != nullptr;
+    const bool ok = major == 10 && minor == 3 && encode_fn() != nullptr;
+    at.store(ok ? 2 : 1, std::memory_order_relaxed);
+    return ok;
 }
 
 

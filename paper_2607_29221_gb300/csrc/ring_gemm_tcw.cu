@@ -576,7 +576,7 @@ mosaic_status ring_gemm_tcw(const uint32_t *A, int64_t lda, const uint32_t *B, i
     if (!make_w_map(&tw, B, K, N, ldb) || !make_x_map(&tx, Ap, K, M, Kp, nt)) return MOSAIC_ERR_CUDA;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+        (sms = sm_count(dev)) < 1)
         return MOSAIC_ERR_CUDA;
     const int64_t tiles = (N + WR - 1) / WR, nst = (K + KS - 1) / KS, nchunks = (nst + CHUNK - 1) / CHUNK;
     if (tiles * nchunks > (int64_t)INT32_MAX) return MOSAIC_ERR_SHAPE;

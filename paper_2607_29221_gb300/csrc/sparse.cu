@@ -525,12 +525,18 @@ mosaic_status launch_pgather(const GatherArgs &a, cudaStream_t st) {
     const size_t smem = pgather_smem(a.r);
     auto kern = pgather_kernel<LIST_IS_COL, CLAMP>;
     static std::atomic<unsigned long long> attr_set{0};   // one bit per device ordinal
-    int dev = 0, sms = 0, per_sm = 0;
-    if (!ensure_smem_limit(attr_set, kern, 227 * 1024, &dev)) return MOSAIC_ERR_CUDA;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPgWarps * 32, smem) != cudaSuccess ||
-        per_sm < 1)
-        return MOSAIC_ERR_CUDA;
+    int dev = 0, sms = 0;
+    if (!ensure_smem_limit(attr_set, kern, 227 * 1024, &dev) || (sms = sm_count(dev)) < 1) return MOSAIC_ERR_CUDA;
+    // Resident CTAs per SM for this stage size, looked up once (32-position steps, per device ordinal).
+    static std::atomic<signed char> occupancy[64][kPgMaxR / 32 + 1];
+    std::atomic<signed char> &known = occupancy[dev & 63][(a.r + 31) / 32];
+    int per_sm = known.load(std::memory_order_relaxed);
+    if (per_sm < 1) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPgWarps * 32, smem) != cudaSuccess ||
+            per_sm < 1)
+            return MOSAIC_ERR_CUDA;
+        known.store((signed char)per_sm, std::memory_order_relaxed);
+    }
     const int64_t tiles = (a.g_count + kPgRows - 1) / kPgRows;
     const int64_t tiles2 = a.two ? (a.g_count2 + kPgRows - 1) / kPgRows : 0;
     const int64_t chunks = (a.nlist + kPgEnts - 1) / kPgEnts;
@@ -625,7 +631,7 @@ mosaic_status launch_few(const GatherArgs &a, cudaStream_t st) {
     static std::atomic<unsigned long long> attr_set{0};   // one bit per device ordinal
     int dev = 0, sms = 0;
     if (!ensure_smem_limit(attr_set, kern, 192 * 1024, &dev) ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        (sms = sm_count(dev)) < 1)
         return MOSAIC_ERR_CUDA;
     // Enough warps to stream the lists; every block stages the rows once.
     const int64_t need = (a.nlist + kFewWarps - 1) / kFewWarps;

@@ -334,7 +334,7 @@ mosaic_status launch(Kernel kern, std::atomic<unsigned long long> &attr_set, int
                      int per_sm, cudaStream_t st) {
     int dev = 0, sms = 0;
     if (!ensure_smem_limit(attr_set, kern, kUnmaskFewSmem, &dev) ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+        (sms = sm_count(dev)) < 1)
         return MOSAIC_ERR_CUDA;
     const int need = (a.m + kUfWarps * rows - 1) / (kUfWarps * rows);
     const int slots = sms * per_sm;

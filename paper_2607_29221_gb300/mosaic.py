@@ -177,6 +177,8 @@ def _stream(stream):
     if stream is not None:
         return stream if isinstance(stream, int) else stream.cuda_stream
     import torch
+    if torch.cuda.is_initialized():   # the raw handle, without a Stream object per call
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     return torch.cuda.current_stream().cuda_stream
 
 

@@ -561,6 +561,153 @@ mosaic_status launch_pgather(const GatherArgs &a, cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------------------
+// Direct gather: the same sums straight from the tile images in global memory,
+// every level in one launch.  A warp takes one list entity and one tile, a
+// lane one row; position p's 32 rows are one 128-byte line of the image, so a
+// (position, value) pair is one coalesced line load that the L1 cache serves
+// when the SM's other warps touched the line (a block's 32 warps walk
+// consecutive entities of one tile).  Against the staged gather it saves the
+// copy of whole 128-192 KB images per CTA and level, one launch and one pass
+// over the outputs per level, and it splits the work by 32 entities instead
+// of 128; it loses where many entities share a tile, since every pair then
+// also costs its list reads by the whole warp.
+//
+// It is taken up to kDirectTasks (entity, tile) pairs, or, with the entities as
+// output rows (Init X), up to kDirectEnts entities whatever the tiles.
+// Measured, whole call, staged -> direct, microseconds: unmask of 64 tokens x
+// 128 outputs (256 pairs) 35 -> 24, 64 x 4096 (8192) 37.2 -> 35.0, 96 x 4096
+// (12288) 51.6 -> 57.5; Init X of 8192 + 8192 rows, 5 tokens 111 -> 60, 32 tokens
+// 122 -> 95, 64 tokens 124 -> 126; of 8192 + 57344 rows, 32 tokens 373 -> 303, 64
+// tokens 375 -> 425; of 1024 + 1024 rows, 128 tokens (8192) 52.2 -> 50.7, 192
+// tokens (12288) 53.5 -> 58.9.
+// ---------------------------------------------------------------------------
+constexpr int kDgWarps = 32;
+constexpr int64_t kDirectTasks = 8192, kDirectEnts = 48;
+
+struct DirectArgs {
+    const uint32_t *img[2], *img2[2];   // per level: images of the first and the second job
+    const uint32_t *idx[2], *val[2];
+    int t[2], rp[2], lines[2];
+    uint32_t rlast[2];
+    int nlev;
+    int64_t nlist, g_count, g_count2;   // second job: its tiles follow the first's (0 rows: none)
+    const uint32_t *a;
+    int64_t lda;
+    uint32_t *out, *out2;               // rows = entities; nullable for columns
+    int64_t ldo, ldo2;
+    const float *s_w, *s_x, *bias;
+    float *Y;
+    int64_t ldy;
+};
+
+// COL = false: out[e][g] += sum (both jobs).  COL = true: entity e is an output
+// column, row g a token: Y_hat = a[g][e] - sum, then decode.
+template <bool COL>
+__global__ void __launch_bounds__(kDgWarps * 32, 1) dgather_kernel(DirectArgs a, int groups, int units) {
+    __shared__ uint32_t tr[COL ? 32 : 1][33];
+    pdl_enter();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t tiles1 = (a.g_count + kPgRows - 1) / kPgRows;
+    const int u_begin = (int)((int64_t)units * blockIdx.x / gridDim.x);
+    const int u_end = (int)((int64_t)units * (blockIdx.x + 1) / gridDim.x);
+    int64_t tile = u_begin / groups;
+    int grp = u_begin % groups;
+    for (int u = u_begin; u < u_end; u++) {
+        const bool second = !COL && tile >= tiles1;
+        const int64_t tl = second ? tile - tiles1 : tile;
+        const int64_t e = (int64_t)grp * kDgWarps + warp;
+        const int64_t g = tl * kPgRows + lane;
+        uint32_t s0 = 0u, s1 = 0u, s2 = 0u, s3 = 0u;
+        if (e < a.nlist) {
+#pragma unroll
+            for (int L = 0; L < 2; L++) {
+                if (L >= a.nlev) break;
+                const char *base = reinterpret_cast<const char *>(second ? a.img2[L] : a.img[L]) +
+                                   (size_t)tl * (size_t)a.rp[L] * 128u;
+                const uint4 *ip = reinterpret_cast<const uint4 *>(a.idx[L] + e * a.t[L]);
+                const uint4 *vp = reinterpret_cast<const uint4 *>(a.val[L] + e * a.t[L]);
+                const int quads = a.t[L] >> 2;
+                const uint32_t rlast = a.rlast[L];
+                const bool lines = a.lines[L] != 0;
+#pragma unroll 5
+                for (int q = 0; q < quads; q++) {
+                    uint4 I = ip[q];
+                    const uint4 V = vp[q];
+                    if (!lines)
+                        I = make_uint4(pg_line(min(I.x, rlast)), pg_line(min(I.y, rlast)), pg_line(min(I.z, rlast)),
+                                       pg_line(min(I.w, rlast)));
+                    // A line offset carries its chunk permutation in bits 4..6, so the
+                    // XOR with 4 lane is the byte of row `lane`.
+                    s0 += V.x * *reinterpret_cast<const uint32_t *>(base + (I.x ^ (uint32_t)(4 * lane)));
+                    s1 += V.y * *reinterpret_cast<const uint32_t *>(base + (I.y ^ (uint32_t)(4 * lane)));
+                    s2 += V.z * *reinterpret_cast<const uint32_t *>(base + (I.z ^ (uint32_t)(4 * lane)));
+                    s3 += V.w * *reinterpret_cast<const uint32_t *>(base + (I.w ^ (uint32_t)(4 * lane)));
+                }
+            }
+        }
+        const uint32_t sum = s0 + s1 + s2 + s3;
+        if (!COL) {
+            if (e < a.nlist && g < (second ? a.g_count2 : a.g_count)) {
+                uint32_t *o = (second ? a.out2 : a.out) + e * (second ? a.ldo2 : a.ldo) + g;
+                *o += sum;
+            }
+        } else {
+            // 32 entities x 32 rows change places so that a row's 32 columns go out together.
+            tr[lane][warp] = sum;
+            __syncthreads();
+            const int64_t row = tl * kPgRows + warp, col = (int64_t)grp * kDgWarps + lane;
+            if (row < a.g_count && col < a.nlist) {
+                const uint32_t res = a.a[row * a.lda + col] - tr[warp][lane];
+                if (a.out) a.out[row * a.ldo + col] = res;
+                float y = __fmul_rn(__fmul_rn(__int2float_rn((int32_t)res), a.s_w[col]), a.s_x[row]);
+                if (a.bias) y = __fadd_rn(y, a.bias[col]);
+                a.Y[row * a.ldy + col] = y;
+            }
+            __syncthreads();
+        }
+        if (++grp == groups) {
+            grp = 0;
+            ++tile;
+        }
+    }
+}
+
+// Whether the direct gather takes these levels (images of every segment, lists
+// that load as quads) and is the better of the two for the size.
+bool direct_ok(bool list_is_col, int64_t tiles, int64_t nlist, const SparseLevel *lev, int nlev) {
+    if (nlev < 1 || nlev > kMaxLev) return false;
+    for (int L = 0; L < nlev; L++)
+        if (!lev[L].tiled || lev[L].t < 4 || lev[L].t % 4 || lev[L].r < 1 || !aligned16(lev[L].idx) || !aligned16(lev[L].val))
+            return false;
+    return tiles * nlist <= kDirectTasks || (!list_is_col && nlist <= kDirectEnts);
+}
+
+void direct_levels(DirectArgs &d, const SparseLevel *lev, int nlev) {
+    d.nlev = nlev;
+    for (int L = 0; L < nlev; L++) {
+        d.img[L] = lev[L].tiled;
+        d.idx[L] = lev[L].idx; d.val[L] = lev[L].val;
+        d.t[L] = lev[L].t; d.rp[L] = (int)((lev[L].r + 31) / 32 * 32);
+        d.lines[L] = lev[L].lines; d.rlast[L] = lev[L].r - 1;
+    }
+}
+
+template <bool COL>
+mosaic_status launch_direct(const DirectArgs &a, cudaStream_t st) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || (sms = sm_count(dev)) < 1) return MOSAIC_ERR_CUDA;
+    const int64_t tiles = (a.g_count + kPgRows - 1) / kPgRows + (a.g_count2 + kPgRows - 1) / kPgRows;
+    const int64_t groups = (a.nlist + kDgWarps - 1) / kDgWarps, units = tiles * groups;
+    if (units > 0x7fffffff) return MOSAIC_ERR_SHAPE;
+    {
+        KernelSpan span("dgather", st);
+        pdl_launch(dgather_kernel<COL>, (unsigned)(units < sms ? units : sms), kDgWarps * 32, 0, st, a, (int)groups,
+                   (int)units);
+    }
+    return launch_status();
+}
+
+// ---------------------------------------------------------------------------
 // Few staged rows (g_count <= 4, e.g. the unmask of a decode step): one warp
 // per list entity.  Each block stages the g_count rows of the level's segment
 // once and its warps walk entities; the 32 lanes read an entity's (position,
@@ -1129,6 +1276,20 @@ mosaic_status sparse_gather_pair(const uint32_t *src, int64_t lds, int64_t g_cou
     }
     if (g_count == 0 && g_count2 == 0) return MOSAIC_OK;
     if (nlist == 0) return MOSAIC_OK;
+    SparseLevel with_img[kMaxLev];
+    for (int L = 0; L < nlev; L++) {
+        with_img[L] = lev[L];
+        with_img[L].tiled = img[L];
+    }
+    if (direct_ok(false, (g_count + kPgRows - 1) / kPgRows + (g_count2 + kPgRows - 1) / kPgRows, nlist, with_img,
+                  nlev)) {
+        DirectArgs d{};
+        direct_levels(d, with_img, nlev);
+        for (int L = 0; L < nlev; L++) d.img2[L] = img2[L];
+        d.nlist = nlist; d.g_count = g_count; d.g_count2 = g_count2;
+        d.out = out; d.ldo = ldo; d.out2 = out2; d.ldo2 = ldo2;
+        return launch_direct<false>(d, st);
+    }
     for (int L = 0; L < nlev; L++) {
         GatherArgs g{};
         g.src = src; g.lds = lds; g.g_count = g_count; g.nlist = nlist;
@@ -1151,6 +1312,14 @@ mosaic_status unmask_decode(const uint32_t *Z, int64_t ldz, int64_t seg_off, int
                             const float *bias, float *Y, uint32_t *Yhat, int64_t ldy,
                             cudaStream_t st, bool folded) {
     (void)seg_off; (void)seg_len;
+    if (folded && l > 0 && m > 0 && direct_ok(true, (l + kPgRows - 1) / kPgRows, m, lev, nlev)) {
+        DirectArgs d{};
+        direct_levels(d, lev, nlev);
+        d.nlist = m; d.g_count = l;
+        d.a = tmp; d.lda = ldt; d.out = Yhat; d.ldo = ldy;
+        d.s_w = s_w; d.s_x = s_x; d.bias = bias; d.Y = Y; d.ldy = ldy;
+        return launch_direct<true>(d, st);
+    }
     GatherArgs g{};
     g.src = Z; g.lds = ldz; g.g_count = l; g.nlist = m;
     if (folded) {

@@ -565,3 +565,14 @@ def test_prg_uniform_quads(rows, cols, ld, off):
     got = host_u32(out)
     assert np.array_equal(got[:, :cols], O.sample_uniform(KEY, tg, sid, rows, cols, 20))
     assert np.all(got[:, cols:] == 0xFFFFFFFF)
+
+
+# Direct and staged gathers on both sides of where one takes over: 48 / 49 entities with many tiles
+# (Init X), 8190 / 8193 (entity, tile) pairs (unmask), one-level and two-level lists, ragged rows.
+@pytest.mark.parametrize("d,r,t,m,l", [
+    (3, (96, 64, 40), (8, 4), 6000, 48), (3, (96, 64, 40), (8, 4), 6000, 49), (3, (96, 64, 40), (8, 4), 2730, 96),
+    (3, (96, 64, 40), (8, 4), 2731, 96), (2, (96, 40), (12,), 77, 33), (3, (100, 70, 36), (20, 16), 133, 95),
+    (3, (1536, 1024, 652), (80, 80), 65, 40), (3, (1536, 1024, 652), (80, 80), 31, 6)])
+def test_gathers_direct_and_staged(d, r, t, m, l):
+    g, ref, op, m, l = _run_layer(d, r, t, m=m, n=100, l=l, variant=M_().GEMM_AUTO)
+    _check_layer(g, ref, op, m, l)

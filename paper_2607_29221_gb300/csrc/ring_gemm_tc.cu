@@ -123,7 +123,7 @@ struct TcArgs {
     int64_t ldc2;
     const uint32_t *Cin2;
     int64_t ldcin2;
-    // Plain mode, first output: C = Cin - Csub + sgn * A B^T (Csub nullable).
+    // First output: C = Cin - Csub + sgn * A B^T (Csub nullable).
     const uint32_t *Csub;
     int64_t ldcsub;
 };
@@ -618,15 +618,33 @@ struct TcOut {
     const uint32_t *Cin;
     int64_t ldcin;
     int64_t cols;
-    const uint32_t *Csub = nullptr;   // first output only, plain mode
+    const uint32_t *Csub = nullptr;   // first output only
     int64_t ldcsub = 0;
 };
 
+// C = Cin - Csub over [c0, cols) of every row (blockIdx.y): the start of a
+// shared output with a subtracted input.
+__global__ void start_diff_kernel(uint32_t *C, int64_t ldc, const uint32_t *Cin, int64_t ldcin, const uint32_t *Csub,
+                                  int64_t ldcsub, int64_t c0, int64_t cols, int64_t rows) {
+    pdl_trigger();
+    const int64_t c = c0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= cols) return;
+    for (int64_t r = blockIdx.y; r < rows; r += gridDim.y)
+        C[r * ldc + c] = (Cin ? Cin[r * ldcin + c] : 0u) - Csub[r * ldcsub + c];
+}
+
 // Prepares the columns [c0, cols) of a stream-K output, whose tiles are (or
-// may be) summed with atomic adds: they start as Cin (or 0).
+// may be) summed with atomic adds: they start as Cin (or 0), less Csub.
 cudaError_t prepare_split(const TcOut &o, int64_t M, int64_t c0, cudaStream_t st) {
     if (c0 < 0) c0 = 0;
     if (o.cols <= c0) return cudaSuccess;
+    if (o.Csub) {
+        KernelSpan span("start_diff", st);
+        start_diff_kernel<<<dim3((unsigned)((o.cols - c0 + 255) / 256), (unsigned)(M < 1024 ? M : 1024)), 256, 0, st>>>(
+            o.C, o.ldc, o.Cin, o.ldcin, o.Csub, o.ldcsub, c0, o.cols, M);
+        count_launch();
+        return cudaPeekAtLastError();
+    }
     const size_t width = (size_t)(o.cols - c0) * 4;
     if (!o.Cin) return cudaMemset2DAsync(o.C + c0, (size_t)o.ldc * 4, 0, width, (size_t)M, st);
     if (o.Cin != o.C)
@@ -663,8 +681,12 @@ mosaic_status launch_tc(const uint16_t *Ap, int64_t ldpa, int64_t a_plane, const
     // 1536, 6 chunks, 256 tiles: 91.5 us whole, 87 us split; 3 chunks: 56
     // against 33 us.)
     const int64_t waves = (tiles + sms - 1) / sms;
-    // A subtracted input is read in plain mode only (stream-K prepares C from Cin alone).
-    const bool split = !o1.Csub && nchunks >= 6 && (double)tiles / (double)(waves * sms) < 0.9;
+    // With few tiles, though, K is split where that takes two chunks or more off
+    // every CTA: the time of a small grid is the time of its longest K walk
+    // (64 x 384 x 652, 3 tiles: 25 -> 13 us).
+    const int64_t share = (tiles * nchunks + sms - 1) / sms;   // chunks of the busiest CTA when split
+    const bool split = (nchunks >= 6 && (double)tiles / (double)(waves * sms) < 0.9) ||
+                       (waves == 1 && nchunks - share >= 2);
     TcArgs args{Cm, ldc, Cin, ldcin, sgn, (int)M, (int)N, (int)K, (int)tiles_m, (int)tiles_n, split ? 1 : 0,
                 0, (int)o1.cols, o2.C, o2.ldc, o2.Cin, o2.ldcin, o1.Csub, o1.ldcsub};
     int64_t grid = tiles < sms ? tiles : sms;

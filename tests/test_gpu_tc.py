@@ -298,3 +298,13 @@ def test_few_tokens_tile_heights(Mm, N):
                        N, Mm, N, K, M.GEMM_TC, None)
     M.mosaic_device_status()
     assert np.array_equal(host(C), ref(A, B))
+
+
+# Few tiles of 2 to 5 chunks: K is split over idle SMs where that saves two chunks or more (one tile;
+# 50 and 51 tiles of 3 chunks, on both sides of a second chunk per CTA), ragged rows and K tails.
+@pytest.mark.parametrize("Mm,N,K", [(65, 130, 652), (100, 128, 513), (70, 6400, 652), (70, 6401, 652), (300, 700, 1100),
+                                    (129, 3000, 1030), (65, 256, 300)])
+def test_tc_few_tiles_split_k(Mm, N, K):
+    A = wl.uniform_u32(171, Mm, K)
+    B = wl.uniform_u32(172, N, K)
+    assert np.array_equal(ring_gemm_u32(A, B), ref(A, B))

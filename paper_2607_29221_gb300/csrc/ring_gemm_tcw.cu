@@ -139,17 +139,28 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t *v) {
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// Digit i of two elements (already offset by 0x80808080) as two fp16 values
-// (byte - 128) in one word: the bytes sit in the mantissas of 1024 + byte,
+// Digits of two elements (already offset by 0x80808080) as fp16 values
+// (byte - 128), digit i of both in word d[i]: the bytes are interleaved once,
+// then one permutation per digit puts them into the mantissas of 1024 + byte
 // and one packed subtraction of 1152 leaves byte - 128 (exact: every value
-// involved is an integer below 2^11).
-__device__ __forceinline__ uint32_t digit_pair_f16(uint32_t b0, uint32_t b1, int i) {
-    const uint32_t t = __byte_perm(b0, b1, (uint32_t)i | ((uint32_t)(4 + i) << 8));
-    const uint32_t h = (t & 0x00FF00FFu) | 0x64006400u;
-    __half2 x = *reinterpret_cast<const __half2 *>(&h);
+// involved is an integer below 2^11).  12 instructions a pair with the offset
+// adds; a permutation and a masked OR per digit took 14, and the ALU is what
+// bounds the kernel (60556 x 8192, 32 tokens: 406 -> 378 us; without the
+// digits 322, without the products 339; sixteen converter warps, or the digits
+// ahead of the slot's wait, gave nothing).
+__device__ __forceinline__ void digit_pairs_f16(uint32_t b0, uint32_t b1, uint32_t &d0, uint32_t &d1, uint32_t &d2,
+                                                uint32_t &d3) {
+    const uint32_t lo = __byte_perm(b0, b1, 0x5140), hi = __byte_perm(b0, b1, 0x7362);   // b0_0 b1_0 b0_1 b1_1, ...
+    const uint32_t h[4] = {__byte_perm(lo, 0x64646464u, 0x4140), __byte_perm(lo, 0x64646464u, 0x4342),
+                           __byte_perm(hi, 0x64646464u, 0x4140), __byte_perm(hi, 0x64646464u, 0x4342)};
     const uint32_t c = 0xE480E480u;   // (-1152, -1152)
-    x = __hadd2(x, *reinterpret_cast<const __half2 *>(&c));
-    return *reinterpret_cast<uint32_t *>(&x);
+    uint32_t r[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const __half2 x = __hadd2(*reinterpret_cast<const __half2 *>(&h[i]), *reinterpret_cast<const __half2 *>(&c));
+        r[i] = *reinterpret_cast<const uint32_t *>(&x);
+    }
+    d0 = r[0]; d1 = r[1]; d2 = r[2]; d3 = r[3];
 }
 
 // Exact fold of the four shift groups of one column into acc (mod 2^32).
@@ -362,12 +373,13 @@ __global__ void __launch_bounds__(THREADS, 1)
                 }
                 fence_after();
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    uint32_t d[16];
+                for (int h = 0; h < 2; ++h) {   // 16 K: 8 words of every plane
+                    uint32_t d[4][8];
 #pragma unroll
-                    for (int p = 0; p < 16; ++p) d[p] = digit_pair_f16(w[2 * p], w[2 * p + 1], i);
-                    tmem_st8(lane_base + (uint32_t)(b * SLOT_COLS + 32 * i), d);
-                    tmem_st8(lane_base + (uint32_t)(b * SLOT_COLS + 32 * i + 8), d + 8);
+                    for (int p = 0; p < 8; ++p)
+                        digit_pairs_f16(w[16 * h + 2 * p], w[16 * h + 2 * p + 1], d[0][p], d[1][p], d[2][p], d[3][p]);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) tmem_st8(lane_base + (uint32_t)(b * SLOT_COLS + 32 * i + 8 * h), d[i]);
                 }
                 tmem_st_wait();
                 fence_before();

@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(kPgWarps * 32, 1)
                 if (it < total && g0 + g < g_count && p < r) {
                     const uint32_t *srow = src + (g0 + g) * lds + a.col0;
                     if (vec_src && p + 4 <= r) {
-                        w[j] = *reinterpret_cast<const uint4 *>(srow + p);
+                        w[j] = __ldca(reinterpret_cast<const uint4 *>(srow + p));
                     } else {
                         w[j].x = srow[p];
                         if (p + 1 < r) w[j].y = srow[p + 1];
@@ -423,11 +423,11 @@ __global__ void __launch_bounds__(kPgWarps * 32, 1)
 #pragma unroll
                 for (int h = 0; h < 2; h++) {
                     if (ja) {
-                        const uint4 x = *reinterpret_cast<const uint4 *>(ja + e * jlda + g + 4 * h);
+                        const uint4 x = __ldca(reinterpret_cast<const uint4 *>(ja + e * jlda + g + 4 * h));
                         ab[4 * h] = x.x; ab[4 * h + 1] = x.y; ab[4 * h + 2] = x.z; ab[4 * h + 3] = x.w;
                     }
                     if (a.b) {
-                        const uint4 x = *reinterpret_cast<const uint4 *>(a.b + e * a.ldb + g + 4 * h);
+                        const uint4 x = __ldca(reinterpret_cast<const uint4 *>(a.b + e * a.ldb + g + 4 * h));
                         ab[4 * h] -= x.x; ab[4 * h + 1] -= x.y; ab[4 * h + 2] -= x.z; ab[4 * h + 3] -= x.w;
                     }
                 }
@@ -608,14 +608,23 @@ __global__ void __launch_bounds__(kDgWarps * 32, 1) dgather_kernel(DirectArgs a,
     pdl_enter();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t tiles1 = (a.g_count + kPgRows - 1) / kPgRows;
+    const int64_t tiles = tiles1 + (a.g_count2 + kPgRows - 1) / kPgRows;
     const int u_begin = (int)((int64_t)units * blockIdx.x / gridDim.x);
     const int u_end = (int)((int64_t)units * (blockIdx.x + 1) / gridDim.x);
-    int64_t tile = u_begin / groups;
-    int grp = u_begin % groups;
     for (int u = u_begin; u < u_end; u++) {
+        // COL: a unit is 32 entities of one tile.  Else it is 32 consecutive (tile,
+        // entity) pairs, so that a few entities still fill the block's warps.
+        int64_t tile, e;
+        if (COL) {
+            tile = u / groups;
+            e = (int64_t)(u - (int)tile * groups) * kDgWarps + warp;
+        } else {
+            const int64_t pair = (int64_t)u * kDgWarps + warp;
+            tile = pair / a.nlist;
+            e = tile < tiles ? pair - tile * a.nlist : a.nlist;
+        }
         const bool second = !COL && tile >= tiles1;
         const int64_t tl = second ? tile - tiles1 : tile;
-        const int64_t e = (int64_t)grp * kDgWarps + warp;
         const int64_t g = tl * kPgRows + lane;
         uint32_t s0 = 0u, s1 = 0u, s2 = 0u, s3 = 0u;
         if (e < a.nlist) {
@@ -655,7 +664,7 @@ __global__ void __launch_bounds__(kDgWarps * 32, 1) dgather_kernel(DirectArgs a,
             // 32 entities x 32 rows change places so that a row's 32 columns go out together.
             tr[lane][warp] = sum;
             __syncthreads();
-            const int64_t row = tl * kPgRows + warp, col = (int64_t)grp * kDgWarps + lane;
+            const int64_t row = tl * kPgRows + warp, col = e - warp + lane;
             if (row < a.g_count && col < a.nlist) {
                 const uint32_t res = a.a[row * a.lda + col] - tr[warp][lane];
                 if (a.out) a.out[row * a.ldo + col] = res;
@@ -664,10 +673,6 @@ __global__ void __launch_bounds__(kDgWarps * 32, 1) dgather_kernel(DirectArgs a,
                 a.Y[row * a.ldy + col] = y;
             }
             __syncthreads();
-        }
-        if (++grp == groups) {
-            grp = 0;
-            ++tile;
         }
     }
 }
@@ -697,7 +702,8 @@ mosaic_status launch_direct(const DirectArgs &a, cudaStream_t st) {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || (sms = sm_count(dev)) < 1) return MOSAIC_ERR_CUDA;
     const int64_t tiles = (a.g_count + kPgRows - 1) / kPgRows + (a.g_count2 + kPgRows - 1) / kPgRows;
-    const int64_t groups = (a.nlist + kDgWarps - 1) / kDgWarps, units = tiles * groups;
+    const int64_t groups = (a.nlist + kDgWarps - 1) / kDgWarps;
+    const int64_t units = COL ? tiles * groups : (tiles * a.nlist + kDgWarps - 1) / kDgWarps;
     if (units > 0x7fffffff) return MOSAIC_ERR_SHAPE;
     {
         KernelSpan span("dgather", st);

@@ -673,20 +673,17 @@ mosaic_status launch_tc(const uint16_t *Ap, int64_t ldpa, int64_t a_plane, const
     if (tiles * nchunks > (int64_t)INT32_MAX) return MOSAIC_ERR_SHAPE;   // 32-bit unit numbers
     const int sms = sm_count(dev);
     if (sms < 1) return MOSAIC_ERR_CUDA;
-    // Whole tiles on a persistent grid (at most one CTA per SM) unless the
-    // last wave would leave more than 10% of the SMs idle; then the grid also
-    // shares the remaining tiles' (tile, chunk) units evenly.  Short products
-    // (fewer than 6 chunks) keep whole tiles only: there the preparation of C
-    // and the split-tile atomics cost more than the idle SMs.  (512 x 8192 x
-    // 1536, 6 chunks, 256 tiles: 91.5 us whole, 87 us split; 3 chunks: 56
-    // against 33 us.)
-    const int64_t waves = (tiles + sms - 1) / sms;
-    // With few tiles, though, K is split where that takes two chunks or more off
-    // every CTA: the time of a small grid is the time of its longest K walk
-    // (64 x 384 x 652, 3 tiles: 25 -> 13 us).
-    const int64_t share = (tiles * nchunks + sms - 1) / sms;   // chunks of the busiest CTA when split
-    const bool split = (nchunks >= 6 && (double)tiles / (double)(waves * sms) < 0.9) ||
-                       (waves == 1 && nchunks - share >= 2);
+    // Whole tiles on a persistent grid (at most one CTA per SM), or, where that
+    // takes two 256-K chunks or more off the busiest CTA, whole waves of tiles
+    // and the remaining tiles' (tile, chunk) units shared evenly (a chunk is 7
+    // us of tensor work; preparing the shared columns and their atomic adds
+    // cost about 6 us a launch).  2048 x 13452 x 8192 (1696 tiles, 384 -> 358
+    // chunks): 2.59 -> 2.43 ms; 512 x 8192 x 1536 (256 tiles, 12 -> 11): 91.5 us
+    // whole, 87 us split; 64 x 384 x 652 (3 tiles, 3 -> 1): 25 -> 13 us.
+    const int64_t waves = (tiles + sms - 1) / sms, rest = tiles % sms;
+    const int64_t whole_chunks = waves * nchunks;
+    const int64_t split_chunks = tiles / sms * nchunks + (rest * nchunks + sms - 1) / sms;
+    const bool split = whole_chunks - split_chunks >= (nchunks >= 6 ? 1 : 2);
     TcArgs args{Cm, ldc, Cin, ldcin, sgn, (int)M, (int)N, (int)K, (int)tiles_m, (int)tiles_n, split ? 1 : 0,
                 0, (int)o1.cols, o2.C, o2.ldc, o2.Cin, o2.ldcin, o1.Csub, o1.ldcsub};
     int64_t grid = tiles < sms ? tiles : sms;

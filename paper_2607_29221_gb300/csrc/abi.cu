@@ -837,12 +837,9 @@ mosaic_status unmask_impl(const mosaic_params *p, int64_t l, int64_t m, const ui
         lev[i - 1] = SparseLevel{S_idx + soff, S_val + soff, (int)t, m + off_r(p, i), ri};
         soff += m * t;
     }
-    // Up to 16 tokens everything runs in one launch, which reads L and the S
-    // lists once (70B gate+up at one token: 80 us as a product and two gathers).
-    if (want_tc && unmask_few_ok(l, m, rd, (int)d - 1, lev))
-        return unmask_few(l, m, Z, ldz, m + od, rd, K_tm, L, (int)d - 1, lev, s_w, s_x, bias, Y, Yhat, ldy, st);
     const int64_t Kp = kpad8(rd);
-    const bool room = cv.used + up(8 * (size_t)(l * Kp)) <= cv.cap;
+    const size_t planes = up(8 * (size_t)(l * Kp));
+    const bool room = cv.used + planes <= cv.cap;
     // Up to kTcwMaxM tokens the product streams the uint32 L (half the bytes of
     // its planes, and a token tile of its own size; whole unmask at 32 tokens,
     // 57344 rows: 146 -> 113 us, 8192: 49.6 -> 40.1 us); more take L's planes.
@@ -853,6 +850,13 @@ mosaic_status unmask_impl(const mosaic_params *p, int64_t l, int64_t m, const ui
     // from planes; AUTO is the fastest for the shape.
     const bool stream_l = (variant == MOSAIC_GEMM_AUTO || !Lp) && want_tc && tc_available() && room && l <= kTcwMaxM &&
                           l >= kTcwMinM && rd % 4 == 0 && aligned16(L);
+    // Up to 16 tokens everything runs in one launch, which reads L and the S
+    // lists once (70B gate+up at one token: 80 us as a product and two gathers),
+    // unless it is better to stream L even then.
+    if (want_tc && unmask_few_ok(l, m, rd, (int)d - 1, lev) &&
+        !(stream_l && cv.used + planes + unmask_images_bytes(l, p) <= cv.cap &&
+          unmask_few_loses(l, m, rd, (int)d - 1, lev)))
+        return unmask_few(l, m, Z, ldz, m + od, rd, K_tm, L, (int)d - 1, lev, s_w, s_x, bias, Y, Yhat, ldy, st);
     const bool tc_planes = !stream_l && Lp && want_tc && !skinny_ok(Qd, ldz, L, rd, l, rd) && room;
     uint16_t *Qp = stream_l || tc_planes ? cv.take<uint16_t>((size_t)(4 * l * Kp)) : nullptr;
     // With room in the workspace, the gathers stage Q_i from tile images made

@@ -24,7 +24,8 @@
 //   before       82.7       113.2      139.4       15.6      33.8      38.5
 //   now          43.0        92.6      140.1        7.9      14.3      22.9
 // (43 us = 5.2 TB/s of L and S lists; at 16 tokens the shared-memory reads
-// and multiply-adds of a row bind instead.)
+// and multiply-adds of a row bind instead: unmask_few_loses() tells where such a
+// call is better off with its rows on the tensor cores, 57344 x 16 in 104 us.)
 #include "mosaic_internal.cuh"
 
 namespace mosaic {
@@ -369,6 +370,30 @@ size_t smem_bytes(int64_t l, int64_t rd, int nlev, const SparseLevel *lev) {
 bool unmask_few_ok(int64_t l, int64_t m, int64_t rd, int nlev, const SparseLevel *lev) {
     return l >= 1 && l <= 16 && m <= (int64_t)INT32_MAX / 2 && nlev <= 2 &&
            smem_bytes(l, rd, nlev, lev) <= kUnmaskFewSmem;
+}
+
+// With 9 to 16 tokens the rows' multiply-adds and shared-memory reads bind, so
+// the time goes up with every round of rows over the warps (32.5, 54, 76, ...
+// us at the Example 3.1 ranks), while the tensor-core product of the same rows
+// is bound by reading them and its gathers by their launches.  It wins from
+// the second round on where a row holds enough words and its lists take the
+// tiled gather.  Whole call at 16 tokens,
+// one launch -> streamed, microseconds, by words a row (r_d + sum of t):
+//   rows     812 (652, 80, 80)   1536 (one level)   732 (652, 80)   280 (200, 40, 40)
+//    8192      33.4 / 38.4          25.1 / 26.5       23.1 / 29.7      16.8 / 24.6
+//   10240      54.1 / 39.6          42.1 / 31.1       37.5 / 28.1      25.1 / 27.5
+//   20480      76.3 / 62.5          60.1 / 42.4       52.1 / 43.3      36.6 / 42.6
+//   57344     144.2 / 104.0        115.5 / 92.2       98.6 / 73.3      59.2 / 61.8
+constexpr int64_t kFewRowWords = 512;
+bool unmask_few_loses(int64_t l, int64_t m, int64_t rd, int nlev, const SparseLevel *lev) {
+    int64_t words = rd;
+    for (int i = 0; i < nlev; i++) {
+        if (!pgather_takes(l, lev[i].r, lev[i].t) || !aligned16(lev[i].idx) || !aligned16(lev[i].val)) return false;
+        words += lev[i].t;
+    }
+    int dev = 0;
+    return l > 8 && words >= kFewRowWords && cudaGetDevice(&dev) == cudaSuccess &&
+           m > (int64_t)sm_count(dev) * kUfWarps * 4;
 }
 
 mosaic_status unmask_few(int64_t l, int64_t m, const uint32_t *Z, int64_t ldz, int64_t dcol, int64_t rd,

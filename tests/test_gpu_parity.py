@@ -540,6 +540,17 @@ def test_unmask_of_few_tokens(d, r, t, m, l):
     _check_layer(g, ref, op, m, l)
 
 
+# 9 to 16 tokens on both sides of one round of rows over the warps (152 SMs x 16 warps x 4 rows) and of
+# 512 words a row: one launch, or L streamed; and ranks and lists that
+# forbid streaming L or the tiled gather.
+@pytest.mark.parametrize("r,t,m,l", [
+    ((96, 64, 500), (8, 4), 9728, 9), ((96, 64, 500), (8, 4), 9729, 9), ((96, 64, 500), (8, 4), 9803, 16),
+    ((96, 64, 496), (8, 4), 9729, 12), ((96, 64, 501), (8, 4), 9729, 9), ((96, 64, 520), (7, 4), 9729, 9), ((96, 64, 500), (8, 4), 9729, 8)])
+def test_unmask_of_few_tokens_and_many_rows(r, t, m, l):
+    g, ref, op, m, l = _run_layer(3, r, t, m=m, n=40, l=l, variant=M_().GEMM_AUTO)
+    _check_layer(g, ref, op, m, l)
+
+
 # Above 16 tokens: the product that streams L (17 to 64 tokens, each token-tile size) and the one from
 # L's planes (65 up), with odd output widths (every row of Z and Y' unaligned), ragged tiles and
 # ranks that forbid streaming L (37) or leave one K stage.

@@ -16,7 +16,16 @@
 //     CHUNK * BK = 256 values of K (group 3 then holds 1024 products) the
 //     epilogue warps drain groups 2 and 3, every 512 values of K groups 0 and
 //     1, into int32 registers: acc += g_s << 8s mod 2^32 (drain_01 and
-//     drain_23 below convert the fp32 sums exactly).
+//     fold_23 below convert the fp32 sums exactly).
+// The tensor pipe does not wait for a drain: the two pairs of groups have
+// products and barriers of their own and are drained half a chunk apart, the
+// pair to be drained goes first in the stage before and second in the stage
+// after, so the other pair's products of two stages (768 clocks beside a drain
+// of groups 2 and 3, 1792 beside 0 and 1) cover the epilogue's round trip
+// without holding a stage back.  With all four groups waiting for each drain:
+// 512 x 7308 x 4096 188.0 -> 182.5 us (1630 -> 1679 TFLOP/s of digit products),
+// 2048 x 13452 x 8192 2456 -> 2395 (1838 -> 1885), 4096 x 3212 x 4096 668.7 ->
+// 656.2; under the power limit (2048 x 60556 x 8192) the same within 0.3%.
 //
 // Pipeline (128 x BN output tiles, 18 warps):
 //   warp 0      TMA producer: per stage one 3-D box {32 K, rows, 4 planes}
@@ -184,9 +193,9 @@ __global__ void __launch_bounds__(THREADS, 1)
                                                 ~static_cast<uintptr_t>(1023));
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + STAGES * C::STAGE);
     uint64_t *empty = full + STAGES;
-    uint64_t *acc_full = empty + STAGES;
-    uint64_t *acc_empty = acc_full + 1;
-    uint64_t *drain = acc_empty + 1;
+    uint64_t *acc_full = empty + STAGES;   // [0]: groups 0 and 1, [1]: groups 2 and 3
+    uint64_t *acc_empty = acc_full + 2;
+    uint64_t *drain = acc_empty + 2;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drain + 1);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
     const uint32_t epi_base = smem_u32(smem + STAGES * C::STAGE + 256);
@@ -216,12 +225,16 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     const int n_units = n0 + n1;
     // Shift groups 0 and 1 gather 1 and 2 digit products per K value, so they
-    // stay exact (|sum| <= 2^24) over two 256-wide chunks and are drained every
-    // second chunk of a tile (and at the end of the tile or of a segment);
-    // groups 2 and 3 are drained after every chunk.  `since` counts the chunks
-    // accumulated in groups 0 and 1, including the current one.
-    auto drains01 = [&](int k, int c, int since) {
-        return since >= 2 || c == nchunks - 1 || k == n0 - 1 || k == n_units - 1;
+    // stay exact (|sum| <= 2^24) over 512 K = 2 CHUNK stages; groups 2 and 3 are
+    // drained after every chunk.  The drains of groups 0 and 1 lie in the
+    // middle of a chunk, after its stage MID - 1, and at the end of a segment of
+    // a tile (where all four are drained).  `since` counts the stages in groups
+    // 0 and 1 before the chunk: at most 12, and 4 right after a middle drain.
+    constexpr int MID = CHUNK / 2;
+    auto seg_end = [&](int k, int c) { return c == nchunks - 1 || k == n0 - 1 || k == n_units - 1; };
+    auto chunk_stages = [&](int c) { return (c + 1) * CHUNK < nk ? CHUNK : nk - c * CHUNK; };
+    auto mid_drain = [&](int since, int nst, bool last) {
+        return nst > MID && since >= CHUNK && !(last && since + nst <= 2 * CHUNK);
     };
     // Walks this CTA's units in order without divisions: (tile, chunk c) of
     // unit k (segment 0: tiles blockIdx.x + w * gridDim.x; segment 1: units
@@ -251,8 +264,10 @@ __global__ void __launch_bounds__(THREADS, 1)
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
-        mbar_init(acc_full, 1);
-        mbar_init(acc_empty, EPI_WARPS);
+        for (int g = 0; g < 2; ++g) {
+            mbar_init(&acc_full[g], 1);
+            mbar_init(&acc_empty[g], EPI_WARPS);
+        }
         mbar_init(drain, 1);
         *abort_flag = 0;
         mbar_init_fence();
@@ -311,27 +326,24 @@ __global__ void __launch_bounds__(THREADS, 1)
     } else if (warp == 1) {
         if (lane == 0) {
             bool issued_any = false;
-            uint32_t chunk_count = 0;
+            uint32_t drains[2] = {0u, 0u};        // drains asked for, per pair of groups
+            bool busy[2] = {false, false};        // the last of them may still be going on
+            bool fresh[2] = {true, true};         // the pair's next product starts its sums
             int s = 0;          // shared-memory slot of the next stage
             uint32_t ph = 0;    // parity of its full barrier
-            int since01 = 0;
+            int since = 0;
             // Descriptors differ only in the start-address field (address >> 4).
             const uint64_t desc0 = sdesc_sw64(smem_u32(smem));
             constexpr uint64_t AP = C::A_PLANE >> 4, BP = C::B_PLANE >> 4;
             UnitWalk w;
             walk_init(w);
             for (; w.k < n_units && !*abort_flag; walk_next(w)) {
-                const int k = w.k;
-                const int c = w.c;
-                const int ks0 = c * CHUNK, ks1 = (c + 1) * CHUNK < nk ? (c + 1) * CHUNK : nk;
-                const uint32_t keep01 = since01 > 0 ? 1u : 0u;   // groups 0, 1 carry on
-                if (drains01(k, c, ++since01)) since01 = 0;
-                if (chunk_count > 0 && !mbar_wait(acc_empty, (uint32_t)(chunk_count - 1) & 1, abort_flag)) {
-                    raise_abort(abort_flag);
-                    break;
-                }
+                const bool last = seg_end(w.k, w.c);
+                const int nst = chunk_stages(w.c);
+                const bool mid = mid_drain(since, nst, last);
+                since = last ? 0 : mid ? nst - MID : since + nst;
                 bool ok = true;
-                for (int ks = ks0; ks < ks1; ++ks) {
+                for (int j = 0; j < nst && ok; ++j) {
                     if (!mbar_wait(&full[s], ph, abort_flag)) {
                         raise_abort(abort_flag);
                         ok = false;
@@ -340,25 +352,51 @@ __global__ void __launch_bounds__(THREADS, 1)
                     tc_fence_after();
                     const uint64_t da = desc0 + (uint64_t)((s * C::STAGE) >> 4);
                     const uint64_t db = da + (uint64_t)(C::A_BYTES >> 4);
-                    const bool first = ks == ks0;
+                    const bool end = j == nst - 1;
+                    // Which pairs are drained once this stage's products are in.
+                    const bool ask[2] = {(mid && j == MID - 1) || (end && last), end};
                     // The 10 digit products d_i e_j (i + j <= 3) as 6 MMAs: B planes
                     // j and j + 1 are adjacent in shared memory and the shift
                     // groups i + j and i + j + 1 adjacent in TMEM, so one N = 2 BN
-                    // product covers both.  A plane 0 goes first: its two paired
-                    // products start all four groups of a chunk.
-#pragma unroll
-                    for (int kk = 0; kk < BK / 16; ++kk) {
-                        const uint32_t z = (first && kk == 0) ? 0u : 1u;
-                        const uint32_t z01 = (first && kk == 0) ? keep01 : 1u;
-                        const uint64_t a0 = da + 2 * kk, b0 = db + 2 * kk;
-                        umma_bf16(tmem + 0 * BN, a0, b0, C::IDESC2, z01);             // d0 e0, d0 e1
-                        umma_bf16(tmem + 2 * BN, a0, b0 + 2 * BP, C::IDESC2, z);      // d0 e2, d0 e3
-                        umma_bf16(tmem + 1 * BN, a0 + AP, b0, C::IDESC2, 1u);         // d1 e0, d1 e1
-                        umma_bf16(tmem + 3 * BN, a0 + AP, b0 + 2 * BP, C::IDESC, 1u); // d1 e2
-                        umma_bf16(tmem + 2 * BN, a0 + 2 * AP, b0, C::IDESC2, 1u);     // d2 e0, d2 e1
-                        umma_bf16(tmem + 3 * BN, a0 + 3 * AP, b0, C::IDESC, 1u);      // d3 e0
-                    }
+                    // product covers both.  No product writes both a group of 0, 1
+                    // and one of 2, 3, so that one pair's products run while the
+                    // other is drained: the pair that is drained after this stage
+                    // goes first, the pair that is being drained goes second.
+                    const bool high_first = (busy[0] && !busy[1]) || (end && !last);
                     issued_any = true;
+                    auto pair = [&](const int g) {   // g is a constant once inlined
+                        if (busy[g]) {
+                            if (!mbar_wait(&acc_empty[g], (drains[g] - 1) & 1, abort_flag)) {
+                                raise_abort(abort_flag);
+                                return false;
+                            }
+                            tc_fence_after();
+                            busy[g] = false;
+                        }
+#pragma unroll
+                        for (int kk = 0; kk < BK / 16; ++kk) {
+                            const uint32_t z = fresh[g] && kk == 0 ? 0u : 1u;
+                            const uint64_t a0 = da + 2 * kk, b0 = db + 2 * kk;
+                            if (g == 0) {
+                                umma_bf16(tmem + 0 * BN, a0, b0, C::IDESC2, z);                   // d0 e0, d0 e1
+                                umma_bf16(tmem + 1 * BN, a0 + AP, b0, C::IDESC, 1u);              // d1 e0
+                            } else {
+                                umma_bf16(tmem + 2 * BN, a0, b0 + 2 * BP, C::IDESC2, z);          // d0 e2, d0 e3
+                                umma_bf16(tmem + 2 * BN, a0 + AP, b0 + BP, C::IDESC2, 1u);        // d1 e1, d1 e2
+                                umma_bf16(tmem + 2 * BN, a0 + 2 * AP, b0, C::IDESC2, 1u);         // d2 e0, d2 e1
+                                umma_bf16(tmem + 3 * BN, a0 + 3 * AP, b0, C::IDESC, 1u);          // d3 e0
+                            }
+                        }
+                        fresh[g] = ask[g];
+                        if (ask[g]) {
+                            umma_commit(&acc_full[g]);
+                            ++drains[g];
+                            busy[g] = true;
+                        }
+                        return true;
+                    };
+                    ok = high_first ? pair(1) && pair(0) : pair(0) && pair(1);
+                    if (!ok) break;
                     umma_commit(&empty[s]);
                     if (++s == STAGES) {
                         s = 0;
@@ -366,8 +404,6 @@ __global__ void __launch_bounds__(THREADS, 1)
                     }
                 }
                 if (!ok) break;
-                umma_commit(acc_full);
-                ++chunk_count;
             }
             if (*abort_flag && issued_any) {
                 // Products in flight still read shared memory and write TMEM.
@@ -389,25 +425,26 @@ __global__ void __launch_bounds__(THREADS, 1)
         uint32_t acc[HB];
 #pragma unroll
         for (int c = 0; c < HB; ++c) acc[c] = 0u;
-        uint32_t chunk_count = 0;
-        int since01 = 0;
+        uint32_t taken[2] = {0u, 0u};   // drains done, per pair of groups
+        int since = 0;
         UnitWalk wk;
         walk_init(wk);
         for (; wk.k < n_units; walk_next(wk)) {
             const int k = wk.k, tile = wk.tile;
             const int c = wk.c;
-            if (!mbar_wait(acc_full, (uint32_t)chunk_count & 1, abort_flag)) {
-                raise_abort(abort_flag);
-                break;
-            }
-            tc_fence_after();
-            const bool d01 = drains01(k, c, ++since01);
-            if (d01) since01 = 0;
-            // Two groups are loaded before one wait.  Groups 2 and 3 are folded
-            // into one fp32 value as they are loaded; its conversion follows
-            // once the accumulators are handed back, beside the next chunk's
-            // products.
-            if (d01) {
+            const bool last = seg_end(k, c);
+            const int nst = chunk_stages(c);
+            const bool mid = mid_drain(since, nst, last);
+            since = last ? 0 : mid ? nst - MID : since + nst;
+            // Groups 0 and 1, in the middle of the chunk, at its end, or both.
+            bool ok = true;
+            for (int e = (mid ? 1 : 0) + (last ? 1 : 0); e > 0; --e) {
+                if (!mbar_wait(&acc_full[0], taken[0] & 1, abort_flag)) {
+                    raise_abort(abort_flag);
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
 #pragma unroll
                 for (int c0 = 0; c0 < HB; c0 += 16) {
                     uint32_t v0[16], v1[16];
@@ -417,7 +454,20 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
                     for (int cc = 0; cc < 16; ++cc) acc[c0 + cc] += drain_01(v0[cc], v1[cc]);
                 }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&acc_empty[0]);
+                ++taken[0];
             }
+            if (!ok) break;
+            if (!mbar_wait(&acc_full[1], taken[1] & 1, abort_flag)) {
+                raise_abort(abort_flag);
+                break;
+            }
+            tc_fence_after();
+            // Groups 2 and 3 are folded into one fp32 value as they are loaded; its
+            // conversion follows once the accumulators are handed back, beside
+            // the next products.
             float s23[HB];
 #pragma unroll
             for (int c0 = 0; c0 < HB; c0 += 16) {
@@ -430,10 +480,10 @@ __global__ void __launch_bounds__(THREADS, 1)
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(acc_empty);
+            if (lane == 0) mbar_arrive(&acc_empty[1]);
 #pragma unroll
             for (int cc = 0; cc < HB; ++cc) acc[cc] += (uint32_t)__float2int_rn(s23[cc]) << 16;
-            ++chunk_count;
+            ++taken[1];
 
             // Short products (no stream-K): one chunk before the tile is written,
             // pull this lane's row of the added / subtracted inputs into L2, so
@@ -461,7 +511,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 }
             }
 
-            if (c != nchunks - 1 && k != n0 - 1 && k != n_units - 1) continue;
+            if (!last) continue;
             // End of this CTA's segment of the tile: write it out.
             const bool whole = k < n0 || ((s1b <= tile * nchunks) && (c == nchunks - 1));
             const int m0 = (int)(tile % a.tiles_m) * BM;
@@ -556,18 +606,18 @@ __global__ void __launch_bounds__(THREADS, 1)
                         }
                         const int gr0 = m0 + q * 32 + i0 + (lane >> 4);
                         if (col >= nout || gr0 >= a.M) continue;
-                        const int last = a.M - 1;
+                        const int rlast = a.M - 1;
                         if (!atomic) {
                             uint32_t x[4];
                             if (cin0) {
 #pragma unroll
-                                for (int u = 0; u < 4; ++u) x[u] = cin0[(int64_t)min(gr0 + 2 * u, last) * ldcin_o + col];
+                                for (int u = 0; u < 4; ++u) x[u] = cin0[(int64_t)min(gr0 + 2 * u, rlast) * ldcin_o + col];
 #pragma unroll
                                 for (int u = 0; u < 4; ++u) v[u] += x[u];
                             }
                             if (sub0) {
 #pragma unroll
-                                for (int u = 0; u < 4; ++u) x[u] = sub0[(int64_t)min(gr0 + 2 * u, last) * a.ldcsub + col];
+                                for (int u = 0; u < 4; ++u) x[u] = sub0[(int64_t)min(gr0 + 2 * u, rlast) * a.ldcsub + col];
 #pragma unroll
                                 for (int u = 0; u < 4; ++u) v[u] -= x[u];
                             }
@@ -575,7 +625,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
                             const int gr = gr0 + 2 * u;
-                            if (gr > last) continue;
+                            if (gr > rlast) continue;
                             uint32_t *const cp = cbase + (int64_t)gr * ldc_o + col;
                             if (atomic) atomicAdd(cp, v[u]);
                             else *cp = v[u];

@@ -308,3 +308,18 @@ def test_tc_few_tiles_split_k(Mm, N, K):
     A = wl.uniform_u32(171, Mm, K)
     B = wl.uniform_u32(172, N, K)
     assert np.array_equal(ring_gemm_u32(A, B), ref(A, B))
+
+
+@pytest.mark.parametrize("Mm,N", [(128, 128), (1600, 1500)])
+@pytest.mark.parametrize("stages", [1, 4, 5, 8, 9, 12, 13, 16, 17, 20, 21, 24, 25, 28, 29, 33, 45])
+def test_tc_drain_points(Mm, N, stages):
+    """Every place of the two drains in a tile's last chunk (K of 1 to 45 stages
+    of 32), one tile shared by CTAs and whole tiles one after another, with
+    all digits -128: a sum kept one stage too long leaves fp32's integers."""
+    for K in (32 * stages, 32 * stages - 27):
+        A = np.full((Mm, K), ALL_M128, np.uint32)
+        B = np.full((N, K), ALL_M128, np.uint32)
+        A[::3, ::5] = 0x01020304
+        B[::2, ::7] = 0xFEDCBA98
+        want = ref(A[:2], B[:2])[np.ix_(np.minimum(np.arange(Mm) % 3, 1), np.arange(N) % 2)]
+        assert np.array_equal(tc_gemm(A, B), want), K

@@ -127,11 +127,11 @@ __global__ void __launch_bounds__(GW * 32) gather_kernel(GatherArgs a) {
     if (t == 0) {
         for (int k = 0; k < n_ent; k++) finish(e_first + (int64_t)k * stride, 0u);
     } else if (vec) {
-        // Rounds of 16 (position, value) pairs.  Lanes 0 .. 8 EPW - 1 copy the
-        // warp's next round into a 2-slot shared-memory ring (cp.async,
-        // zero-filled past the end of a list or of the entity range) while
-        // the current round is gathered; the TG lanes of an entity read its
-        // pairs from the ring with broadcast loads.
+        // Rounds of 16 (position, value) pairs.  The warp's lanes copy the next
+        // round of its EPW entities (8 parts of 16 bytes each) into a 2-slot
+        // shared-memory ring (cp.async, zero-filled past the end of a list or of
+        // the entity range) while the current round is gathered; the TG lanes
+        // of an entity read its pairs from the ring with broadcast loads.
         const int R = (t + 15) >> 4;
         const int steps = n_ent * R;
         uint32_t *ring = sg + ((int64_t)TG * a.segp + 3) / 4 * 4 + warp * (kRing * 32 * EPW);
@@ -140,17 +140,20 @@ __global__ void __launch_bounds__(GW * 32) gather_kernel(GatherArgs a) {
         auto issue = [&](int s) {
             const int k = ik, rr = ir;
             if (++ir == R) { ir = 0; ++ik; }
-            if (lane < 8 * EPW && s < steps) {
-                const int he = lane >> 3, part = lane & 7;
-                const int64_t e = e_begin + warp * EPW + he + (int64_t)k * stride;
-                const int q = rr * 16 + (part & 3) * 4;
-                const bool ok = e < e_end && q < t;
-                const uint32_t *src = (part < 4 ? a.idx : a.val) + (ok ? e * t + q : 0);
-                const uint32_t dst =
-                    (uint32_t)__cvta_generic_to_shared(ring + ((s % kRing) * EPW + he) * 32 + part * 4);
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
-                             "r"(ok ? 16 : 0)
-                             : "memory");
+            if (s < steps) {
+#pragma unroll
+                for (int c = lane; c < 8 * EPW; c += 32) {   // EPW > 4: several parts a lane
+                    const int he = c >> 3, part = c & 7;
+                    const int64_t e = e_begin + warp * EPW + he + (int64_t)k * stride;
+                    const int q = rr * 16 + (part & 3) * 4;
+                    const bool ok = e < e_end && q < t;
+                    const uint32_t *src = (part < 4 ? a.idx : a.val) + (ok ? e * t + q : 0);
+                    const uint32_t dst =
+                        (uint32_t)__cvta_generic_to_shared(ring + ((s % kRing) * EPW + he) * 32 + part * 4);
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
+                                 "r"(ok ? 16 : 0)
+                                 : "memory");
+                }
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
         };

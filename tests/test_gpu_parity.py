@@ -587,3 +587,13 @@ def test_prg_uniform_quads(rows, cols, ld, off):
 def test_gathers_direct_and_staged(d, r, t, m, l):
     g, ref, op, m, l = _run_layer(d, r, t, m=m, n=100, l=l, variant=M_().GEMM_AUTO)
     _check_layer(g, ref, op, m, l)
+
+
+# Segments that leave room for only 4, 2 or 1 staged rows a block (the gather of ranks above 1536 words),
+# so that a warp serves 8, 16 or 32 list entities and copies several parts of their lists a lane;
+# two list rounds, the second one ragged.
+@pytest.mark.parametrize("d,r,t", [(3, (3200, 3100, 64), (20, 12)), (2, (7000, 64), (20,)), (2, (13000, 48), (20,)),
+                                   (2, (20500, 40), (20,))])
+def test_gather_of_large_ranks(d, r, t):
+    g, ref, op, m, l = _run_layer(d, r, t, m=70, n=40, l=37, variant=M_().GEMM_AUTO)
+    _check_layer(g, ref, op, m, l)

@@ -260,7 +260,8 @@ int mosaic_gemm_variant_available(int variant);
  * small decode batch) and 8 M ceil8(K) bytes of `ws` for A's digit planes
  * (required above MOSAIC_SKINNY_MAX_M) they run a tensor-core kernel that also
  * reads each element of B once as uint32 and splits it into digits on the
- * chip.  Every path gives the same ring product. */
+ * chip, unless B is small and M at most MOSAIC_SKINNY_MAX_M.  Every path gives
+ * the same ring product. */
 #define MOSAIC_SKINNY_MAX_M 16
 #define MOSAIC_STREAMW_MAX_M 64
 mosaic_status mosaic_ring_gemm(const uint32_t *A, int64_t lda, const uint32_t *B, int64_t ldb,

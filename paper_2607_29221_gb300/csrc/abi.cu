@@ -396,8 +396,9 @@ mosaic_status mosaic_ring_gemm(const uint32_t *A, int64_t lda, const uint32_t *B
         return ring_gemm_mma_s8(A, lda, B, ldb, C, ldc, nullptr, 0, 1, M, N, K, ws, ws_bytes, st);
     if (!tc_available()) return MOSAIC_ERR_UNSUPPORTED;
     Carve cv = carve(ws, ws_bytes);
-    // kTcwMinM .. kTcwMaxM tokens: tensor cores, B read once as uint32 and split on the chip.
-    if (tcw_ok(A, lda, B, ldb, M, N, K)) {
+    // kTcwMinM .. kTcwMaxM tokens: tensor cores, B read once as uint32 and split on the chip
+    // (up to kSkinnyMaxM of them where that beats the CUDA-core streaming kernel).
+    if (tcw_ok(A, lda, B, ldb, M, N, K) && (M > kSkinnyMaxM || tcw_beats_skinny(N, K))) {
         uint16_t *Ap = cv.take<uint16_t>(tcw_ws_bytes(M, K) / 2);
         if (Ap) return ring_gemm_tcw(A, lda, B, ldb, C, ldc, nullptr, 0, nullptr, 0, 1, M, N, K, Ap, st);
         if (M > kSkinnyMaxM) return MOSAIC_ERR_WORKSPACE;

@@ -276,11 +276,13 @@ mosaic_status skinny_status();
 // (16-byte aligned bases, row strides multiples of 4 words, a Blackwell device).
 // From 9 tokens it beats the CUDA-core streaming product, whose multiply-adds
 // then bind (60556 x 8192, one call: 391 against 568 us at 16 tokens, 390
-// against 320 at 8).
+// against 320 at 8), unless the work is small (tcw_beats_skinny).
 constexpr int64_t kTcwMinM = 9;
 constexpr int64_t kTcwMaxM = 64;
 size_t tcw_ws_bytes(int64_t M, int64_t K);
 bool tcw_ok(const uint32_t *A, int64_t lda, const uint32_t *B, int64_t ldb, int64_t M, int64_t N, int64_t K);
+// Whether it is the faster of the two for 9 to 16 tokens.
+bool tcw_beats_skinny(int64_t N, int64_t K);
 mosaic_status ring_gemm_tcw(const uint32_t *A, int64_t lda, const uint32_t *B, int64_t ldb, uint32_t *C,
                             int64_t ldc, const uint32_t *Cin, int64_t ldcin, const uint32_t *Csub, int64_t ldcsub,
                             int sgn, int64_t M, int64_t N, int64_t K, uint16_t *Ap, cudaStream_t st);

@@ -565,6 +565,20 @@ bool tcw_ok(const uint32_t *A, int64_t lda, const uint32_t *B, int64_t ldb, int6
            ldb % 4 == 0 && tc_available();
 }
 
+// Two launches (token split, product) and a pipeline through TMEM: about 8 us
+// however small the work is, where one wave of the streaming kernel's tiles (60
+// rows a CTA) takes about 2.5 us and 1.3 for every 128 of K.  So the line lies at
+// K = 1024, or at a second wave.  16 tokens, one call inside a CUDA graph,
+// streaming kernel -> this one, microseconds:
+//   rows \ K       64           256           512          1024         2048
+//   1024       2.9 / 5.2     3.6 / 7.8     5.1 /  7.9    7.9 /  7.9   13.3 /  7.9
+//   8192       3.7 / 5.4     5.0 / 8.0     7.6 /  8.1   12.8 / 11.7   23.3 / 18.9
+//   16384      5.8 / 5.6     8.4 / 8.2    13.5 / 11.8   23.9 / 19.0   46.2 / 31.9
+bool tcw_beats_skinny(int64_t N, int64_t K) {
+    int dev = 0;
+    return K >= 1024 || (cudaGetDevice(&dev) == cudaSuccess && N > 60 * (int64_t)sm_count(dev));
+}
+
 mosaic_status ring_gemm_tcw(const uint32_t *A, int64_t lda, const uint32_t *B, int64_t ldb, uint32_t *Cm,
                             int64_t ldc, const uint32_t *Cin, int64_t ldcin, const uint32_t *Csub, int64_t ldcsub,
                             int sgn, int64_t M, int64_t N, int64_t K, uint16_t *Ap, cudaStream_t st) {

@@ -266,7 +266,8 @@ def test_mma_s8_adversarial(va, vb):
 @pytest.mark.parametrize("N,K", [(300, 652), (20000 + 77, 1100)])
 def test_few_tokens_with_and_without_workspace(Mm, N, K):
     """9 to 16 tokens stream B through the tensor cores when `ws` holds A's
-    planes and through the CUDA cores when it does not; 17 need the room."""
+    planes and B is not small (here 20077 rows), through the CUDA cores
+    otherwise; 17 need the room."""
     M = _M()
     A = wl.uniform_u32(151 + Mm, Mm, K)
     B = wl.uniform_u32(152, N, K)

@@ -965,10 +965,11 @@ mosaic_status mosaic_freivalds_check(int k, const uint32_t *a, const uint32_t *Y
     if (m < 1 || n_pad < 1 || l < 0 || ldz < m || ldx < n_pad) return MOSAIC_ERR_SHAPE;
     if (l == 0) return MOSAIC_OK;
     if (!a || !Ychk || !Z || !Xp || !bad || !n_bad) return MOSAIC_ERR_ARG;
-    // 2 k l words of ws are part of the call's contract; the one-launch check keeps its sums on the chip.
     Carve cv = carve(ws, ws_bytes);
-    if (!cv.take<uint32_t>((size_t)(k * l)) || !cv.take<uint32_t>((size_t)(k * l))) return MOSAIC_ERR_WORKSPACE;
-    return freivalds_check(k, a, Ychk, m, n_pad, l, Z, ldz, Xp, ldx, bad, n_bad, as_stream(stream));
+    uint32_t *lhs = cv.take<uint32_t>((size_t)(k * l));
+    uint32_t *rhs = cv.take<uint32_t>((size_t)(k * l));
+    if (!lhs || !rhs) return MOSAIC_ERR_WORKSPACE;
+    return freivalds_check(k, a, Ychk, m, n_pad, l, Z, ldz, Xp, ldx, bad, n_bad, lhs, rhs, as_stream(stream));
 }
 
 }  // extern "C"

@@ -2,8 +2,9 @@
 // step 4 and Online step 4; appendix "Computational integrity"):
 //   setup:  Ychk = a W'            (k check vectors, one-time per matrix)
 //   online: a^T Y' == Ychk X'      per token, over Z_{2^32}
-// The online check streams Z and X' once in one launch; the setup's column
-// sums run here too.
+// The online check streams Z and X' once, in one launch for up to about 1200
+// tokens and as two streaming ring products and a comparison beyond; the
+// setup's column sums run here too.
 #include <cooperative_groups.h>
 
 #include "mosaic_internal.cuh"
@@ -58,17 +59,26 @@ __device__ __forceinline__ void dot_rows(uint32_t (&acc)[KV][T], const uint32_t 
 #pragma unroll
             for (int t = 0; t < T; t++)
                 x[t] = t < tn ? __ldcg(reinterpret_cast<const uint4 *>(B + t * ldb + c0) + i) : make_uint4(0u, 0u, 0u, 0u);
+            // From 8 vectors on, the loads of four rows of A are in flight at once: one
+            // after another, their latencies made up most of a share.
+            constexpr int G = KV >= 8 ? 4 : 1;
 #pragma unroll
-            for (int v = 0; v < KV; v++) {
-                if (v >= k) break;
-                const uint4 y = __ldca(reinterpret_cast<const uint4 *>(A + v * lda + c0) + i);
+            for (int v0 = 0; v0 < KV; v0 += G) {
+                if (v0 >= k) break;
+                uint4 y[G];
 #pragma unroll
-                for (int t = 0; t < T; t++) {
-                    mac(v, t, y.x, x[t].x);
-                    mac(v, t, y.y, x[t].y);
-                    mac(v, t, y.z, x[t].z);
-                    mac(v, t, y.w, x[t].w);
-                }
+                for (int g = 0; g < G; g++)
+                    y[g] = G == 1 || v0 + g < k ? __ldca(reinterpret_cast<const uint4 *>(A + (v0 + g) * lda + c0) + i)
+                                                : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+                for (int g = 0; g < G; g++)
+#pragma unroll
+                    for (int t = 0; t < T; t++) {
+                        mac(v0 + g, t, y[g].x, x[t].x);
+                        mac(v0 + g, t, y[g].y, x[t].y);
+                        mac(v0 + g, t, y[g].z, x[t].z);
+                        mac(v0 + g, t, y[g].w, x[t].w);
+                    }
             }
         }
         c = c0 + 4 * quads;
@@ -99,7 +109,7 @@ __device__ __forceinline__ void dot_rows(uint32_t (&acc)[KV][T], const uint32_t 
 // products on 18 blocks each and a comparison took 18.1 + 17.9 + 2.0 us.
 constexpr int kChkThreads = 256;
 template <int KV, int T>
-__global__ void __launch_bounds__(kChkThreads)
+__global__ void __launch_bounds__(kChkThreads, KV >= 8 ? 2 : 4)
     check_kernel(int k, const uint32_t *a, const uint32_t *Ychk, int64_t m, int64_t n_pad, int64_t l,
                  const uint32_t *Z, int64_t ldz, const uint32_t *Xp, int64_t ldx, uint32_t *bad, uint32_t *n_bad,
                  int vec_z, int vec_x) {
@@ -151,13 +161,72 @@ __global__ void __launch_bounds__(kChkThreads)
     cluster.sync();   // the first block has read the others' shared memory
 }
 
+__global__ void compare_kernel(const uint32_t *lhs, const uint32_t *rhs, int k, int64_t l, uint32_t *bad,
+                               uint32_t *n_bad) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= l) return;
+    uint32_t b = 0u;
+    for (int v = 0; v < k; v++) b += lhs[(int64_t)v * l + j] != rhs[(int64_t)v * l + j] ? 1u : 0u;
+    bad[j] = b;
+    if (b) atomicAdd(n_bad, 1u);
+}
+
+// Clusters of S = 2^s blocks of check_kernel<KV, T> that are resident at once on
+// device `dev`, looked up once (0 on failure).
+template <int KV, int T>
+int check_resident(int dev, int s) {
+    static std::atomic<int> cache[64][4];
+    std::atomic<int> &at = cache[dev & 63][s];
+    int n = at.load(std::memory_order_relaxed);
+    if (n > 0) return n;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1u << s);
+    cfg.blockDim = dim3(kChkThreads);
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 1u << s;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, check_kernel<KV, T>, &cfg) != cudaSuccess) return 0;
+    at.store(n, std::memory_order_relaxed);
+    return n;
+}
+
+// The check by one launch of token clusters, or, where their blocks no longer
+// fit on the device at once, by two streaming products (k x l words each in
+// lhs and rhs) and a comparison: every further wave of clusters reads a and
+// Ychk again and leaves no other warps to hide its latencies behind, while the
+// streaming kernel takes 60 tokens a CTA.  From 8 vectors a second wave still
+// pays where the columns are many.  Inside a CUDA graph, microseconds, clusters
+// / products, by k vectors, l tokens and m = n_pad:
+//   m        4, 2048     4, 4096     8, 1024     8, 2048     8, 4096    16, 4096
+//   64      5.1 /  4.8  9.7 /  5.0  5.0 /  5.7   10 /  5.8       -           -
+//   1024    7.0 /  8.7   12 /  9.0  5.9 / 11.7   11 / 11.8   22 / 12.1       -
+//   8192     37 / 38.7   74 / 51.1   19 / 56.5   43 / 58.3   88 / 61.3  151 / 98.6
 template <int KV, int T>
 mosaic_status launch_check(int k, const uint32_t *a, const uint32_t *Ychk, int64_t m, int64_t n_pad, int64_t l,
                            const uint32_t *Z, int64_t ldz, const uint32_t *Xp, int64_t ldx, uint32_t *bad,
-                           uint32_t *n_bad, cudaStream_t st) {
+                           uint32_t *n_bad, uint32_t *lhs, uint32_t *rhs, cudaStream_t st) {
     const int64_t groups = (l + T - 1) / T;
-    int S = 1;
-    while (S < 8 && groups * S < 2 * 152) S *= 2;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || check_resident<KV, T>(dev, 0) < 1) return MOSAIC_ERR_CUDA;
+    const int64_t one = check_resident<KV, T>(dev, 0), waves = (groups + one - 1) / one;
+    if (waves > (KV >= 8 && m + n_pad >= 2048 ? 2 : 1) && skinny_ok(a, m, Z, ldz, k, m) &&
+        skinny_ok(Ychk, n_pad, Xp, ldx, k, n_pad)) {
+        MOSAIC_TRY(ring_gemm_skinny(a, m, Z, ldz, lhs, l, nullptr, 0, 1, k, l, m, st));
+        MOSAIC_TRY(ring_gemm_skinny(Ychk, n_pad, Xp, ldx, rhs, l, nullptr, 0, 1, k, l, n_pad, st));
+        {
+            KernelSpan span("freivalds_compare", st);
+            compare_kernel<<<(unsigned)((l + 255) / 256), 256, 0, st>>>(lhs, rhs, k, l, bad, n_bad);
+        }
+        return launch_status();
+    }
+    // The columns are split over as many blocks as are all resident at once and
+    // have a quad of columns for every thread.
+    int s = 0;
+    while (s < 3 && m + n_pad >= ((int64_t)2048 << s) && groups <= check_resident<KV, T>(dev, s + 1)) ++s;
+    const int S = 1 << s;
     if (groups * S > 0x7fffffff) return MOSAIC_ERR_SHAPE;
     const int vec_z = aligned16(a) && aligned16(Z) && m % 4 == 0 && ldz % 4 == 0;
     const int vec_x = aligned16(Ychk) && aligned16(Xp) && n_pad % 4 == 0 && ldx % 4 == 0;
@@ -207,14 +276,15 @@ mosaic_status freivalds_colsum(const uint32_t *a, int k, const uint32_t *W, int6
 
 mosaic_status freivalds_check(int k, const uint32_t *a, const uint32_t *Ychk, int64_t m, int64_t n_pad,
                               int64_t l, const uint32_t *Z, int64_t ldz, const uint32_t *Xp, int64_t ldx,
-                              uint32_t *bad, uint32_t *n_bad, cudaStream_t st) {
+                              uint32_t *bad, uint32_t *n_bad, uint32_t *lhs, uint32_t *rhs, cudaStream_t st) {
     if (k < 1 || k > kMaxK) return MOSAIC_ERR_ARG;
     if (l == 0) return MOSAIC_OK;
-    // Four tokens a cluster once that still fills the SMs with one cluster of 8 each (l >= 76).
-    const bool four = l >= 76;
+    // Four tokens a cluster once that still fills the SMs with clusters of 8.
+    int dev = 0;
+    const bool four = cudaGetDevice(&dev) == cudaSuccess && 2 * l >= sm_count(dev);
 #define MOSAIC_CHECK(KV)                                                                                         \
-    (four ? launch_check<KV, 4>(k, a, Ychk, m, n_pad, l, Z, ldz, Xp, ldx, bad, n_bad, st)                        \
-          : launch_check<KV, 1>(k, a, Ychk, m, n_pad, l, Z, ldz, Xp, ldx, bad, n_bad, st))
+    (four ? launch_check<KV, 4>(k, a, Ychk, m, n_pad, l, Z, ldz, Xp, ldx, bad, n_bad, lhs, rhs, st)              \
+          : launch_check<KV, 1>(k, a, Ychk, m, n_pad, l, Z, ldz, Xp, ldx, bad, n_bad, lhs, rhs, st))
     if (k <= 2) return MOSAIC_CHECK(2);
     if (k <= 4) return MOSAIC_CHECK(4);
     if (k <= 8) return MOSAIC_CHECK(8);

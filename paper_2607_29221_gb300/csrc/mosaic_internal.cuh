@@ -290,12 +290,12 @@ mosaic_status ring_gemm_tcw(const uint32_t *A, int64_t lda, const uint32_t *B, i
 mosaic_status tcw_status();
 
 // Freivalds check: Y (k x ncols) = a (k x m) W (m x ncols, ldw), and the
-// per-token comparison a^T Y' vs Ychk X'.
+// per-token comparison a^T Y' vs Ychk X' (lhs, rhs: k x l scratch words each).
 mosaic_status freivalds_colsum(const uint32_t *a, int k, const uint32_t *W, int64_t ldw, int64_t m,
                                int64_t ncols, uint32_t *Y, cudaStream_t st);
 mosaic_status freivalds_check(int k, const uint32_t *a, const uint32_t *Ychk, int64_t m, int64_t n_pad,
                               int64_t l, const uint32_t *Z, int64_t ldz, const uint32_t *Xp, int64_t ldx,
-                              uint32_t *bad, uint32_t *n_bad, cudaStream_t st);
+                              uint32_t *bad, uint32_t *n_bad, uint32_t *lhs, uint32_t *rhs, cudaStream_t st);
 
 // Sparse gathers.
 // out[row][col] = a[row][col] - b[row][col] (b nullable) + sgn * sum_lev sum_q val * src[g][off_lev + idx]

@@ -56,3 +56,26 @@ def test_product_of_9_to_16_tokens(kernels, m, waves, dn, K, streamed):
     assert names == ({"split_f16_start", "ring_gemm_tcw"} if streamed else {"ring_gemm_skinny"})
     M.mosaic_ring_gemm(A, K, B, K, want, N, m, N, K, M.GEMM_IMAD)
     assert torch.equal(C, want)
+
+
+# The check: one launch of clusters while their blocks are all resident at once (about 2400 tokens of up to 4
+# vectors, 1200 of more, twice that with many columns), streaming products beyond, where the strides allow them.
+@pytest.mark.parametrize("k,l,m,n,dz,clusters", [
+    (4, 600, 300, 64, 0, True), (4, 5000, 64, 64, 0, False), (3, 5000, 64, 64, 1, True), (16, 1000, 64, 32, 0, True),
+    (16, 2000, 64, 32, 0, False), (9, 2000, 1024, 1024, 0, True), (8, 5000, 1024, 1024, 0, False)])
+def test_check_of_many_tokens(kernels, k, l, m, n, dz, clusters):
+    M = M_()
+    a, Yc, Z, X = (wl.uniform_u32(i, *s) for i, s in enumerate(((k, m), (k, n), (l, m + dz), (l, n))))
+    a[:, :k] = np.eye(k, dtype=np.uint32)
+    Z[:, :k] = X @ Yc.T - Z[:, k:m] @ a[:, k:].T    # honest answers, then every 7th token is tampered with
+    Z[::7, m - 1] += np.uint32(1)                   # an error of 1 shows in every vector whose last entry is not 0
+    want = np.count_nonzero(Z[:, :m] @ a.T != X @ Yc.T, axis=1)
+    dev = lambda x: torch.from_numpy(x.view(np.int32)).cuda()
+    bad, n_bad = empty(l), torch.zeros(1, dtype=torch.int32, device="cuda")
+    w = ws(M.mosaic_workspace_bytes(M.OP_FREIVALDS_CHECK, k, 0, l))
+    args = [dev(x) for x in (a, Yc, Z, X)]
+    names = kernels(lambda: M.mosaic_freivalds_check(k, args[0], args[1], m, n, l, args[2], m + dz, args[3], n, bad,
+                                                     n_bad, w))
+    assert names == ({"freivalds_check"} if clusters else {"ring_gemm_skinny", "freivalds_compare"})
+    assert np.array_equal(bad.cpu().numpy(), want)
+    assert int(n_bad) == np.count_nonzero(want) > 0

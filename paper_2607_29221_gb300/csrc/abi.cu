@@ -848,15 +848,17 @@ mosaic_status unmask_impl(const mosaic_params *p, int64_t l, int64_t m, const ui
     // takes unaligned rows, and the plane product's write-out reads them 64
     // bytes at a time (on the CUDA cores, 301 x 5003 x 652 took 154 us, now 30).
     // A caller that names the TC variant and brings L's planes gets the product
-    // from planes; AUTO is the fastest for the shape.
+    // from planes, unless the one launch below takes the call; AUTO is the
+    // fastest for the shape.
     const bool stream_l = (variant == MOSAIC_GEMM_AUTO || !Lp) && want_tc && tc_available() && room && l <= kTcwMaxM &&
                           l >= kTcwMinM && rd % 4 == 0 && aligned16(L);
     // Up to 16 tokens everything runs in one launch, which reads L and the S
     // lists once (70B gate+up at one token: 80 us as a product and two gathers),
-    // unless it is better to stream L even then.
+    // unless a product that streams L is possible and better even then.
+    const bool streams = l < kTcwMinM ? skinny_ok(Qd, ldz, L, rd, l, rd)
+                                      : stream_l && cv.used + planes + unmask_images_bytes(l, p) <= cv.cap;
     if (want_tc && unmask_few_ok(l, m, rd, (int)d - 1, lev) &&
-        !(stream_l && cv.used + planes + unmask_images_bytes(l, p) <= cv.cap &&
-          unmask_few_loses(l, m, rd, (int)d - 1, lev)))
+        !(streams && unmask_few_loses(l, m, rd, (int)d - 1, lev)))
         return unmask_few(l, m, Z, ldz, m + od, rd, K_tm, L, (int)d - 1, lev, s_w, s_x, bias, Y, Yhat, ldy, st);
     const bool tc_planes = !stream_l && Lp && want_tc && !skinny_ok(Qd, ldz, L, rd, l, rd) && room;
     uint16_t *Qp = stream_l || tc_planes ? cv.take<uint16_t>((size_t)(4 * l * Kp)) : nullptr;

@@ -369,7 +369,7 @@ mosaic_status unmask_decode(const uint32_t *Z, int64_t ldz, int64_t seg_off, int
 // ranks leave room to stage Q in shared memory.
 constexpr size_t kUnmaskFewSmem = 224 * 1024;
 bool unmask_few_ok(int64_t l, int64_t m, int64_t rd, int nlev, const SparseLevel *lev);
-// Whether streaming L through the tensor cores and gathering is the faster of the two.
+// Whether a product that streams L and the gathers are the faster of the two.
 bool unmask_few_loses(int64_t l, int64_t m, int64_t rd, int nlev, const SparseLevel *lev);
 mosaic_status unmask_few(int64_t l, int64_t m, const uint32_t *Z, int64_t ldz, int64_t dcol, int64_t rd,
                          const uint32_t *K_tm, const uint32_t *L, int nlev, const SparseLevel *lev, const float *s_w,

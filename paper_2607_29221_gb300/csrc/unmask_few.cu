@@ -350,11 +350,16 @@ mosaic_status launch_few(const UfArgs &a, size_t smem, cudaStream_t st) {
     static std::atomic<unsigned long long> attr_set{0};   // one bit per device ordinal
     return launch(unmask_few_kernel<NT>, attr_set, 1, a, smem, smem <= 113 * 1024 ? 2 : 1, st);
 }
-// Four rows a warp where that leaves at least one block for most SMs (m >= 64 x 128), else one.
+// Four rows a warp where one row a warp would take three rounds or more over the
+// SMs' warps (4865 rows on 152 SMs), else one.  Ratio of the two, 8 tokens, by
+// (r_d, t, t): rows 2048 4096 6144 8191: (652, 80, 80) 1.65 1.15 0.89 0.73;
+// (1536) 1.59 1.00 0.74 0.59; (64, 8, 8) 1.41 1.07 0.89 0.76.
 template <int CH>
 mosaic_status launch_rows(const UfArgs &a, size_t smem, cudaStream_t st) {
     static std::atomic<unsigned long long> attr1{0}, attr4{0};   // one bit per device ordinal
-    if (a.m >= 8192) return launch(unmask_rows_kernel<CH, 4>, attr4, 4, a, smem, 1, st);
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return MOSAIC_ERR_CUDA;
+    if (a.m > 2 * kUfWarps * sm_count(dev)) return launch(unmask_rows_kernel<CH, 4>, attr4, 4, a, smem, 1, st);
     return launch(unmask_rows_kernel<CH, 1>, attr1, 1, a, smem, 1, st);
 }
 
@@ -372,13 +377,28 @@ bool unmask_few_ok(int64_t l, int64_t m, int64_t rd, int nlev, const SparseLevel
            smem_bytes(l, rd, nlev, lev) <= kUnmaskFewSmem;
 }
 
-// With 9 to 16 tokens the rows' multiply-adds and shared-memory reads bind, so
-// the time goes up with every round of rows over the warps (32.5, 54, 76, ...
-// us at the Example 3.1 ranks), while the tensor-core product of the same rows
-// is bound by reading them and its gathers by their launches.  It wins from
-// the second round on where a row holds enough words and its lists take the
-// tiled gather.  Whole call at 16 tokens,
-// one launch -> streamed, microseconds, by words a row (r_d + sum of t):
+// When the general path (a product that streams L, then the gathers) is the
+// faster one.  It costs about 2 us a launch and a gather pass a level; what it
+// gains lies in the dense words r_d of a row, which the product streams at 7
+// TB/s where the one launch reads L at 5.2 (one or two tokens) or is bound by the
+// shared-memory reads and multiply-adds of its rows (more tokens).  The latter
+// go up with every round of rows over the warps: 2432 rows (152 x 16), and, with
+// four rows a warp from 4865 rows on, 9728.  The lines were drawn through the
+// ratios one launch / general of r_d from 64 to 14000, one to three levels of t
+// = 8, 80, 128 and 400, and 16 to 57344 rows; the lists' words (sum_t = t_2 +
+// t_3) move a line up since the gathers then cost more.  Examples, whole call
+// inside a CUDA graph, one launch / general, microseconds:
+//   1 token, d = 1:  r_d 2048 x 57344 rows 1.00, 4096 x 4096 0.64, 4096 x 57344 1.18
+//   1 token, d = 3, t = 80:  4096 x 57344 0.99, 8192 x 8192 1.15
+//   4 tokens, d = 1:  8192 x 20480 1.14, 12000 x 2448 1.36, 12000 x 1024 0.69
+//   8 tokens, d = 1:  2048 x 4096 1.01, 4096 x 1024 0.74, 4096 x 4096 1.24,
+//                     4096 x 8192 0.94, 4096 x 20480 1.26, 4096 x 28672 0.87
+//   8 tokens, d = 3, t = 80:  4096 x 4096 0.73, 4096 x 12000 1.13
+//   16 tokens, d = 1:  1024 x 2400 0.64, 1536 x 16 1.20, 1536 x 2448 1.38, 2048 x 4864 1.44
+//   16 tokens, d = 3, t = 80:  1536 x 16 0.93, 2700 x 16 1.42, 1536 x 4096 1.08, 2700 x 2448 1.64
+// Beyond 9728 rows, 9 to 16 tokens stream L wherever a row holds enough words
+// (r_d + sum_t); whole call at 16 tokens, one launch -> streamed, microseconds,
+// by words a row:
 //   rows     812 (652, 80, 80)   1536 (one level)   732 (652, 80)   280 (200, 40, 40)
 //    8192      33.4 / 38.4          25.1 / 26.5       23.1 / 29.7      16.8 / 24.6
 //   10240      54.1 / 39.6          42.1 / 31.1       37.5 / 28.1      25.1 / 27.5
@@ -386,14 +406,30 @@ bool unmask_few_ok(int64_t l, int64_t m, int64_t rd, int nlev, const SparseLevel
 //   57344     144.2 / 104.0        115.5 / 92.2       98.6 / 73.3      59.2 / 61.8
 constexpr int64_t kFewRowWords = 512;
 bool unmask_few_loses(int64_t l, int64_t m, int64_t rd, int nlev, const SparseLevel *lev) {
-    int64_t words = rd;
-    for (int i = 0; i < nlev; i++) {
-        if (!pgather_takes(l, lev[i].r, lev[i].t) || !aligned16(lev[i].idx) || !aligned16(lev[i].val)) return false;
-        words += lev[i].t;
-    }
     int dev = 0;
-    return l > 8 && words >= kFewRowWords && cudaGetDevice(&dev) == cudaSuccess &&
-           m > (int64_t)sm_count(dev) * kUfWarps * 4;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    int64_t sum_t = 0;
+    bool tiled = true;   // the general path's gathers take every level in tiles
+    for (int i = 0; i < nlev; i++) {
+        tiled = tiled && pgather_takes(l, lev[i].r, lev[i].t) && aligned16(lev[i].idx) && aligned16(lev[i].val);
+        sum_t += lev[i].t;
+    }
+    const int64_t rows = (int64_t)sm_count(dev) * kUfWarps;   // one row a warp; 4 rows from 2 rounds on
+    if (l <= 2) {
+        if (nlev == 0 && rd < 512) return m > 10 * rows;      // little to read: the rows' own overhead
+        return m * rd >= (int64_t)(nlev ? 20 : 24) << 20 && rd > 2560 + 1024 * nlev;
+    }
+    if (l <= 4) return m > rows && rd > 8192;
+    if (l <= 8) {
+        if (m <= rows) return false;
+        if (m <= 2 * rows) return rd > 2048 + 16 * sum_t;
+        const int64_t rounds = (m + 4 * rows - 1) / (4 * rows);   // the last one may be nearly empty
+        return 2 * m > 9 * rows && m < 3 * rounds * rows && rd > 1792 + 4 * sum_t;
+    }
+    if (!tiled) return false;
+    if (m > 4 * rows) return rd + sum_t >= kFewRowWords;
+    if (m <= rows) return rd > 1280 + 5 * sum_t;
+    return rd > (m <= 2 * rows ? 850 : 1350) + 3 * sum_t;
 }
 
 mosaic_status unmask_few(int64_t l, int64_t m, const uint32_t *Z, int64_t ldz, int64_t dcol, int64_t rd,

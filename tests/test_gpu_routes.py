@@ -79,3 +79,37 @@ def test_check_of_many_tokens(kernels, k, l, m, n, dz, clusters):
     assert names == ({"freivalds_check"} if clusters else {"ring_gemm_skinny", "freivalds_compare"})
     assert np.array_equal(bad.cpu().numpy(), want)
     assert int(n_bad) == np.count_nonzero(want) > 0
+
+
+# The one-launch unmask of up to 16 tokens and the general path (a product that streams L, then gathers) on both sides
+# of each line; `rows` counts rounds of one row a warp (152 SMs x 16 warps). ldz = m + sum(r) + pad.
+@pytest.mark.parametrize("l,r,t,rounds,dm,pad,few", [
+    (1, (4096,), (), 0, 4096, 0, True), (2, (4096,), (), 0, 8192, 0, False), (1, (256,), (), 10, 0, 0, True),
+    (1, (256,), (), 10, 4, 0, False), (2, (96, 64, 8192), (8, 4), 0, 4096, 0, False), (2, (96, 64, 4096), (8, 4), 0, 8192, 0, True),
+    (4, (8196,), (), 1, 0, 0, True), (3, (8196,), (), 1, 4, 0, False), (4, (8192,), (), 1, 4, 0, True),
+    (8, (2052,), (), 1, 0, 0, True), (5, (2052,), (), 1, 4, 0, False), (8, (2052,), (), 2, 0, 1, True),
+    (8, (2048,), (), 2, 0, 0, True), (8, (2052,), (), 2, 4, 0, True), (8, (96, 2052), (40,), 2, 0, 0, True),
+    (8, (1796,), (), 5, 0, 0, False), (8, (1792,), (), 5, 0, 0, True), (8, (1796,), (), 7, 0, 0, True),
+    (16, (1280,), (), 1, 0, 0, True), (9, (1284,), (), 1, 0, 0, False), (12, (848,), (), 1, 4, 0, True),
+    (16, (856,), (), 2, 0, 0, False), (16, (64, 856), (4,), 2, 0, 0, True), (9, (1348,), (), 2, 4, 0, True),
+    (16, (1352,), (), 2, 4, 0, False), (16, (64, 1352), (5,), 2, 4, 0, True)])
+def test_unmask_of_few_tokens(kernels, l, r, t, rounds, dm, pad, few):
+    M = M_()
+    m, d, S = rounds * 16 * sms() + dm, len(r), sum(r)
+    p = M.default_params(d=d, r=r, t=(0,) + t)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    rand = lambda *s: torch.randint(-(1 << 31), 1 << 31, s, generator=g, device="cuda", dtype=torch.int64).to(torch.int32)
+    ldz = m + S + (4 - (m + S)) % 4 + pad
+    Z, K, L, s_w, s_x = rand(l, ldz), rand(l, m), rand(m, r[-1]), torch.rand(m, device="cuda"), torch.rand(l, device="cuda")
+    S_idx = torch.cat([rand(m * t[i]).abs() % r[i] for i in range(d - 1)]) if t else None
+    S_val = rand(m * sum(t)) if t else None
+    w = ws(M.mosaic_workspace_bytes(M.OP_UNMASK, m, 0, l, p))
+    out = {v: (torch.empty(l, m, device="cuda"), empty(l, m)) for v in (M.GEMM_AUTO, M.GEMM_IMAD)}
+    call = lambda v: M.mosaic_unmask(p, l, m, Z, ldz, K, L, S_idx, S_val, s_w, s_x, None, *out[v], m, v, w)
+    names = kernels(lambda: call(M.GEMM_AUTO))
+    if few:
+        assert names == {"unmask_few"}
+    else:
+        assert "unmask_few" not in names and ("ring_gemm_skinny" if l <= 8 else "ring_gemm_tcw") in names
+    call(M.GEMM_IMAD)
+    assert all(torch.equal(a, b) for a, b in zip(out[M.GEMM_AUTO], out[M.GEMM_IMAD]))

@@ -575,17 +575,28 @@ mosaic_status launch_pgather(const GatherArgs &a, cudaStream_t st) {
 // of 128; it loses where many entities share a tile, since every pair then
 // also costs its list reads by the whole warp.
 //
-// It is taken up to kDirectTasks (entity, tile) pairs, or, with the entities as
-// output rows (Init X), up to kDirectEnts entities whatever the tiles.
-// Measured, whole call, staged -> direct, microseconds: unmask of 64 tokens x
-// 128 outputs (256 pairs) 35 -> 24, 64 x 4096 (8192) 37.2 -> 35.0, 96 x 4096
-// (12288) 51.6 -> 57.5; Init X of 8192 + 8192 rows, 5 tokens 111 -> 60, 32 tokens
-// 122 -> 95, 64 tokens 124 -> 126; of 8192 + 57344 rows, 32 tokens 373 -> 303, 64
-// tokens 375 -> 425; of 1024 + 1024 rows, 128 tokens (8192) 52.2 -> 50.7, 192
-// tokens (12288) 53.5 -> 58.9.
+// It is taken for up to one (entity, tile) pair a warp of the device (4864 on 152
+// SMs).  Up to kDirectTasks pairs, warps take two: that still pays with two levels
+// of short lists (one launch and one pass over the outputs less) or very short
+// ones.  With the entities as output rows (Init X) it is also taken up to
+// kDirectEnts entities whatever the tiles, or kDirectEntsPadded where the staged
+// gather's rounds of 16 pairs hold at least a quarter of padding.  Direct /
+// staged, whole call inside a CUDA graph, m outputs, l tokens, by (ranks) and t:
+//                     (1536, 1024, 652)               (512, 64)
+//   t                4    16    80   160   400      4    16    80   160
+//   unmask, m x l
+//   4096 x 32      0.68  0.75  0.67  0.66  0.65   0.82  0.88  0.78  0.75
+//   4096 x 64      0.80  0.93  0.94  1.02  1.13   0.97  1.07  1.05  1.10
+//   Init X of 1024 + 1024 rows
+//   l = 76         0.81  0.85  0.78  0.74    -   0.95  0.98  0.88  0.83
+//   l = 128        0.88  0.95  0.97  1.03  1.12   0.99  1.06  1.06  1.08
+//   Init X of 8192 + 57344 rows
+//   l = 40         0.59  0.89  0.91  0.87  0.80   0.63  1.10  0.81  0.76
+//   l = 48         0.63  0.99  1.01  0.97  0.91   0.70  1.24  0.91  0.89
+//   and l = 48 at t = 12 / 20 / 24 / 32:  0.87 0.77 0.85 1.03, (512, 64) 1.09 0.82 0.94 1.12
 // ---------------------------------------------------------------------------
 constexpr int kDgWarps = 32;
-constexpr int64_t kDirectTasks = 8192, kDirectEnts = 48;
+constexpr int64_t kDirectTasks = 8192, kDirectEnts = 40, kDirectEntsPadded = 48;
 
 struct DirectArgs {
     const uint32_t *img[2], *img2[2];   // per level: images of the first and the second job
@@ -684,10 +695,20 @@ __global__ void __launch_bounds__(kDgWarps * 32, 1) dgather_kernel(DirectArgs a,
 // that load as quads) and is the better of the two for the size.
 bool direct_ok(bool list_is_col, int64_t tiles, int64_t nlist, const SparseLevel *lev, int nlev) {
     if (nlev < 1 || nlev > kMaxLev) return false;
-    for (int L = 0; L < nlev; L++)
+    int longest = 0, pairs = 0, rounds = 0;
+    for (int L = 0; L < nlev; L++) {
         if (!lev[L].tiled || lev[L].t < 4 || lev[L].t % 4 || lev[L].r < 1 || !aligned16(lev[L].idx) || !aligned16(lev[L].val))
             return false;
-    return tiles * nlist <= kDirectTasks || (!list_is_col && nlist <= kDirectEnts);
+        longest = lev[L].t > longest ? lev[L].t : longest;
+        pairs += lev[L].t;
+        rounds += (lev[L].t + 15) / 16;
+    }
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    const int64_t tasks = tiles * nlist;
+    if (tasks <= (int64_t)sm_count(dev) * kDgWarps) return true;
+    if (tasks <= kDirectTasks && longest <= (nlev == 2 ? 80 : 8)) return true;
+    return !list_is_col && nlist <= (4 * pairs <= 3 * 16 * rounds ? kDirectEntsPadded : kDirectEnts);
 }
 
 void direct_levels(DirectArgs &d, const SparseLevel *lev, int nlev) {

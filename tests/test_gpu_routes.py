@@ -113,3 +113,47 @@ def test_unmask_of_few_tokens(kernels, l, r, t, rounds, dm, pad, few):
         assert "unmask_few" not in names and ("ring_gemm_skinny" if l <= 8 else "ring_gemm_tcw") in names
     call(M.GEMM_IMAD)
     assert all(torch.equal(a, b) for a, b in zip(out[M.GEMM_AUTO], out[M.GEMM_IMAD]))
+
+
+# Direct and staged gathers on both sides of each line, for Init X (images of C and J prepared) and the unmask: one
+# (entity, 32-row tile) pair a warp (152 SMs x 32), 8192 pairs with two levels of short lists, 40 or 48 entities.
+@pytest.mark.parametrize("r,t,n_pad,m,l,direct", [
+    ((96, 64, 40), (8, 4), 1024, 1056, 126, True), ((96, 64, 40), (8, 4), 1024, 1056, 127, False),
+    ((200, 180, 40), (80, 84), 1024, 1408, 64, True), ((200, 180, 40), (80, 84), 1024, 1408, 65, False),
+    ((64, 40), (12,), 512, 1920, 64, True), ((64, 40), (12,), 512, 1920, 65, False), ((64, 40), (8,), 512, 1920, 65, True),
+    ((64, 40), (12,), 8192, 6000, 48, True), ((64, 40), (12,), 8192, 6000, 49, False),
+    ((64, 40), (16,), 8192, 6000, 40, True), ((64, 40), (16,), 8192, 6000, 41, False)])
+def test_init_x_gathers(kernels, r, t, n_pad, m, l, direct):
+    M = M_()
+    p, S = M.default_params(d=len(r), r=r, t=(0,) + t), sum(r)
+    key = M.make_key(wl.mask_key())
+    C, J = u32(1, n_pad, S), u32(2, m, S)
+    cj = ws(M.mosaic_workspace_bytes(M.OP_ACTIVATION_PLANES, m, n_pad, 0, p)).view(torch.int16)
+    M.mosaic_prepare_activation(p, m, n_pad, C, J, cj)
+    w = ws(M.mosaic_workspace_bytes(M.OP_MASK_ACTIVATION, m, n_pad, l, p))
+    out = [[empty(l, n_pad), empty(l, m)] for _ in range(2)]
+    names = kernels(lambda: M.mosaic_mask_activation_planes(p, key, 9, m, n_pad, l, C, J, cj, *out[0], M.GEMM_AUTO, w))
+    assert ("dgather" in names, "pgather" in names) == (direct, not direct)
+    M.mosaic_mask_activation(p, key, 9, m, n_pad, l, C, J, *out[1], M.GEMM_IMAD, w)   # no images: staged
+    assert all(torch.equal(a, b) for a, b in zip(*out))
+
+
+@pytest.mark.parametrize("r,t,l,m,direct", [
+    ((96, 64, 40), (8, 4), 96, 2730, True), ((96, 64, 40), (8, 4), 96, 2731, False),
+    ((200, 180, 40), (80, 84), 64, 2432, True), ((200, 180, 40), (80, 84), 64, 2433, False),
+    ((64, 40), (12,), 20, 4864, True), ((64, 40), (12,), 20, 4865, False), ((64, 40), (8,), 20, 4865, True)])
+def test_unmask_gathers(kernels, r, t, l, m, direct):
+    M = M_()
+    p, S, d = M.default_params(d=len(r), r=r, t=(0,) + t), sum(r), len(r)
+    Z, K, L, s_w, s_x = u32(1, l, m + S), u32(2, l, m), u32(3, m, r[-1]), torch.rand(m).cuda(), torch.rand(l).cuda()
+    S_idx = torch.cat([torch.randint(0, r[i], (m * t[i],), dtype=torch.int32) for i in range(d - 1)]).cuda()
+    S_val = u32(4, m, sum(t))
+    Lp = ws(M.mosaic_workspace_bytes(M.OP_UNMASK_PLANES, m, 0, 0, p)).view(torch.int16)
+    M.mosaic_prepare_unmask(p, m, L, Lp)
+    w = ws(M.mosaic_workspace_bytes(M.OP_UNMASK, m, 0, l, p))
+    out = {v: (torch.empty(l, m, device="cuda"), empty(l, m)) for v in (M.GEMM_AUTO, M.GEMM_IMAD)}
+    call = lambda v: M.mosaic_unmask_planes(p, l, m, Z, m + S, K, L, Lp, S_idx, S_val, s_w, s_x, None, *out[v], m, v, w)
+    names = kernels(lambda: call(M.GEMM_AUTO))
+    assert ("dgather" in names, "pgather" in names) == (direct, not direct)
+    assert "dgather" not in kernels(lambda: call(M.GEMM_IMAD))
+    assert all(torch.equal(a, b) for a, b in zip(out[M.GEMM_AUTO], out[M.GEMM_IMAD]))

@@ -177,8 +177,9 @@ def _stream(stream):
     if stream is not None:
         return stream if isinstance(stream, int) else stream.cuda_stream
     import torch
-    if torch.cuda.is_initialized():   # the raw handle, without a Stream object per call
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    raw, device = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+    if raw and device and torch.cuda.is_initialized():   # the raw handle, without a Stream object per call
+        return raw(device())
     return torch.cuda.current_stream().cuda_stream
 
 

@@ -198,3 +198,21 @@ def test_kernel_timing_toggle_without_gpu(lib):
     assert M.mosaic_kernel_timing(True) is False
     assert M.mosaic_kernel_timing(False) is True
     assert M.mosaic_kernel_times(reset=True) == {}
+
+
+@pytest.mark.parametrize("missing", ["_cuda_getCurrentRawStream", "_cuda_getDevice"])
+def test_current_stream_without_torch_internals(monkeypatch, missing):
+    """The raw stream handle comes from torch's private accessors where they
+    exist; a torch without one of them is served by the public call."""
+    torch = pytest.importorskip("torch")
+    from types import SimpleNamespace
+
+    from paper_2607_29221_gb300 import mosaic as M
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: SimpleNamespace(cuda_stream=1234))
+    for name, value in (("_cuda_getCurrentRawStream", lambda dev: 1000 + dev), ("_cuda_getDevice", lambda: 3)):
+        monkeypatch.setattr(torch._C, name, value, raising=False)
+    assert M._stream(None) == 1003
+    monkeypatch.delattr(torch._C, missing)
+    assert M._stream(None) == 1234
+    assert M._stream(77) == 77 and M._stream(SimpleNamespace(cuda_stream=78)) == 78

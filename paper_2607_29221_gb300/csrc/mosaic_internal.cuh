@@ -239,7 +239,8 @@ mosaic_status ring_gemm_tc_planes2(const uint16_t *Ap, int64_t ldpa, int64_t a_p
                                    const uint32_t *Cin1, int64_t ldcin1, int64_t N1, uint32_t *C2, int64_t ldc2,
                                    const uint32_t *Cin2, int64_t ldcin2, int64_t N2, int64_t M, int64_t K,
                                    cudaStream_t st);
-// C = Cin - Csub + sgn * A B^T from planes, one output (K > 0).
+// C = Cin - Csub + sgn * A B^T from planes, one output (K > 0); Cin and Csub
+// must not overlap C (MOSAIC_ERR_ARG when one of them is C).
 mosaic_status ring_gemm_tc_planes_diff(const uint16_t *Ap, int64_t ldpa, int64_t a_plane, const uint16_t *Bp,
                                        int64_t ldpb, int64_t b_plane, uint32_t *C, int64_t ldc,
                                        const uint32_t *Cin, int64_t ldcin, const uint32_t *Csub, int64_t ldcsub,

@@ -808,6 +808,8 @@ mosaic_status ring_gemm_tc_planes_diff(const uint16_t *Ap, int64_t ldpa, int64_t
                                        int sgn, int64_t M, int64_t N, int64_t K, cudaStream_t st) {
     if (M == 0 || N == 0) return MOSAIC_OK;
     if (M > (int64_t)INT32_MAX || N > (int64_t)INT32_MAX || K == 0 || !Cin || !Csub) return MOSAIC_ERR_SHAPE;
+    // Shared columns are prepared as Cin - Csub before whole tiles there read both again.
+    if (Cin == Cm || Csub == Cm) return MOSAIC_ERR_ARG;
     TcOut o1{Cm, ldc, Cin, ldcin, N};
     o1.Csub = Csub;
     o1.ldcsub = ldcsub;

@@ -4,6 +4,7 @@ declares; host-only entry points and argument validation work without a GPU
 import ctypes
 import os
 import re
+import subprocess
 
 import numpy as np
 import pytest
@@ -207,7 +208,6 @@ def test_current_stream_without_torch_internals(monkeypatch, missing):
     torch = pytest.importorskip("torch")
     from types import SimpleNamespace
 
-    from paper_2607_29221_gb300 import mosaic as M
     monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
     monkeypatch.setattr(torch.cuda, "current_stream", lambda: SimpleNamespace(cuda_stream=1234))
     for name, value in (("_cuda_getCurrentRawStream", lambda dev: 1000 + dev), ("_cuda_getDevice", lambda: 3)):
@@ -216,3 +216,20 @@ def test_current_stream_without_torch_internals(monkeypatch, missing):
     monkeypatch.delattr(torch._C, missing)
     assert M._stream(None) == 1234
     assert M._stream(77) == 77 and M._stream(SimpleNamespace(cuda_stream=78)) == 78
+
+
+def test_tc_difference_refuses_its_output_as_an_input(lib):
+    """C = Cin - Csub + A B^T prepares shared columns of C in place, so a C that
+    is also an input would be subtracted from twice: refused before anything
+    is enqueued (called by its C++ name, with addresses that are nothing's, so
+    only where no device could follow them)."""
+    if pytest.importorskip("torch").cuda.is_available():
+        pytest.skip("for hosts without a device")
+    names = subprocess.run(["nm", "-D", "--defined-only", B.LIB], capture_output=True, text=True, check=True).stdout
+    (name,) = re.findall(r"\b(_ZN6mosaic24ring_gemm_tc_planes_diff\w+)", names)
+    f, P, I = getattr(lib, name), ctypes.c_void_p, ctypes.c_int64
+    f.argtypes = [P, I, I, P, I, I, P, I, P, I, P, I, ctypes.c_int, I, I, I, P]
+    f.restype = ctypes.c_int
+    a, b, c, x = 1 << 12, 2 << 12, 3 << 12, 4 << 12
+    for cin, csub in ((c, x), (x, c), (c, c)):
+        assert f(a, 8, 8, b, 8, 8, c, 8, cin, 8, csub, 8, -1, 1, 1, 8, None) == 1   # MOSAIC_ERR_ARG

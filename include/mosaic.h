@@ -290,7 +290,14 @@ mosaic_status mosaic_ring_gemm_planes(const uint16_t *A_planes, int64_t ldpa, in
  *   P  (Sr x n_pad): rows [P_1; P_2; ...; P_d], P_i = M_i ... M_1
  *   C  (n_pad x Sr): columns [C_1 | ... | C_d], C_i = N_1 ... N_i
  *   CT (Sr x n_pad): C transposed.
- * ws: mosaic_workspace_bytes(MOSAIC_OP_MASK_CHAINS, 0, n_pad, 0, p). */
+ * ws: mosaic_workspace_bytes(MOSAIC_OP_MASK_CHAINS, 0, n_pad, 0, p) bytes hold
+ * M_i and N_i (i = 2 .. d) and the digit planes of one product of the chains on
+ * the tensor cores, 8 max_i ((r_i + n_pad) ceil8(r_{i-1})) bytes (default
+ * parameters: 131 MB at n_pad = 8192, 836 MB at 65536).  Any size from M_i and
+ * N_i alone works, sum_i 2 up256(4 r_i r_{i-1}) bytes (up256 rounds up to 256;
+ * 18 MB, plus up to 255 bytes for a ws that is not 256-byte aligned): products
+ * whose planes do not fit run on the CUDA cores, with the same results; less
+ * returns MOSAIC_ERR_WORKSPACE. */
 mosaic_status mosaic_mask_chains(const mosaic_params *p, const mosaic_key *key,
                                  uint64_t chain_id, int64_t n_pad, uint32_t *P, uint32_t *C,
                                  uint32_t *CT, void *ws, size_t ws_bytes, void *stream);

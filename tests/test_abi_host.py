@@ -233,3 +233,18 @@ def test_tc_difference_refuses_its_output_as_an_input(lib):
     a, b, c, x = 1 << 12, 2 << 12, 3 << 12, 4 << 12
     for cin, csub in ((c, x), (x, c), (c, c)):
         assert f(a, 8, 8, b, 8, 8, c, 8, cin, 8, csub, 8, -1, 1, 1, 8, None) == 1   # MOSAIC_ERR_ARG
+
+
+def test_chains_workspace_minimum(lib):
+    """The smallest workspace that the header states for the chains (M_i and
+    N_i alone; with it they run, tests/test_gpu_chains.py): a byte less is refused."""
+    up = lambda v: (v + 255) // 256 * 256
+    for r in ((1536, 1024, 652), (70, 33), (5, 3, 2)):
+        p = M.default_params(d=len(r), r=r, t=(0, 1, 1)[:len(r)])
+        least = sum(2 * up(4 * a * b) for a, b in zip(r, r[1:]))
+        planes = max((b + 8192) * ((a + 7) // 8 * 8) * 8 for a, b in zip(r, r[1:]))
+        assert least + planes <= M.mosaic_workspace_bytes(M.OP_MASK_CHAINS, 0, 8192, 0, p) <= least + planes + 512
+        fake = ctypes.c_void_p(4096)
+        key = M.make_key(range(8))
+        assert lib.mosaic_mask_chains(ctypes.byref(p), ctypes.byref(key), 1, 8192, fake, fake, fake, fake, least - 1,
+                                      None) == 6   # MOSAIC_ERR_WORKSPACE

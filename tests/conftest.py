@@ -11,16 +11,20 @@ if ROOT not in sys.path:
 @pytest.fixture
 def kernels():
     """kernels(call): the names of this library's kernels that call() launched
-    (which of several paths a call took; all of them give the same bits)."""
+    (which of several paths a call took; all of them give the same bits), as a
+    set, or by the entry point's role as {role: set}."""
     from paper_2607_29221_gb300 import mosaic as M
 
-    def run(call):
+    def run(call, by_role=False):
         M.mosaic_kernel_times(reset=True)
         M.mosaic_kernel_timing(True)
         try:
             call()
             M.mosaic_device_status()
-            return {name.split(":")[1] for name in M.mosaic_kernel_times(reset=True)}
+            names = [name.split(":") for name in M.mosaic_kernel_times(reset=True)]
+            if by_role:
+                return {role: {k for r, k in names if r == role} for role, _ in names}
+            return {k for _, k in names}
         finally:
             M.mosaic_kernel_timing(False)
     return run

@@ -540,15 +540,19 @@ def test_unmask_of_few_tokens(d, r, t, m, l):
     _check_layer(g, ref, op, m, l)
 
 
-# 9 to 16 tokens on both sides of one round of rows over the warps (152 SMs x 16 warps x 4 rows) and of
-# 512 words a row: one launch, or L streamed; and ranks and lists that
+# 9 to 16 tokens on both sides of one round of rows over the warps (`over` rows more than 16 warps x 4 rows an SM:
+# 9728 on 152) and of 512 words a row: one launch (`few`), or L streamed; and ranks and lists that
 # forbid streaming L or the tiled gather.
-@pytest.mark.parametrize("r,t,m,l", [
-    ((96, 64, 500), (8, 4), 9728, 9), ((96, 64, 500), (8, 4), 9729, 9), ((96, 64, 500), (8, 4), 9803, 16),
-    ((96, 64, 496), (8, 4), 9729, 12), ((96, 64, 501), (8, 4), 9729, 9), ((96, 64, 520), (7, 4), 9729, 9), ((96, 64, 500), (8, 4), 9729, 8)])
-def test_unmask_of_few_tokens_and_many_rows(r, t, m, l):
-    g, ref, op, m, l = _run_layer(3, r, t, m=m, n=40, l=l, variant=M_().GEMM_AUTO)
-    _check_layer(g, ref, op, m, l)
+@pytest.mark.parametrize("r,t,over,l,few", [
+    ((96, 64, 500), (8, 4), 0, 9, True), ((96, 64, 500), (8, 4), 1, 9, False), ((96, 64, 500), (8, 4), 75, 16, False),
+    ((96, 64, 496), (8, 4), 1, 12, True), ((96, 64, 501), (8, 4), 1, 9, True), ((96, 64, 520), (7, 4), 1, 9, True),
+    ((96, 64, 500), (8, 4), 1, 8, True)])
+def test_unmask_of_few_tokens_and_many_rows(kernels, r, t, over, l, few):
+    m = torch.cuda.get_device_properties(0).multi_processor_count * 64 + over
+    out = []
+    names = kernels(lambda: out.extend(_run_layer(3, r, t, m=m, n=40, l=l, variant=M_().GEMM_AUTO)), by_role=True)["unmask"]
+    assert names == {"unmask_few"} if few else "ring_gemm_tcw" in names and "unmask_few" not in names
+    _check_layer(*out)
 
 
 # Above 16 tokens: the product that streams L (17 to 64 tokens, each token-tile size) and the one from
@@ -578,15 +582,22 @@ def test_prg_uniform_quads(rows, cols, ld, off):
     assert np.all(got[:, cols:] == 0xFFFFFFFF)
 
 
-# Direct and staged gathers on both sides of where one takes over: 48 / 49 entities with many tiles
-# (Init X), 8190 / 8193 (entity, tile) pairs (unmask), one-level and two-level lists, ragged rows.
-@pytest.mark.parametrize("d,r,t,m,l", [
-    (3, (96, 64, 40), (8, 4), 6000, 48), (3, (96, 64, 40), (8, 4), 6000, 49), (3, (96, 64, 40), (8, 4), 2730, 96),
-    (3, (96, 64, 40), (8, 4), 2731, 96), (2, (96, 40), (12,), 77, 33), (3, (100, 70, 36), (20, 16), 133, 95),
-    (3, (1536, 1024, 652), (80, 80), 65, 40), (3, (1536, 1024, 652), (80, 80), 31, 6)])
-def test_gathers_direct_and_staged(d, r, t, m, l):
-    g, ref, op, m, l = _run_layer(d, r, t, m=m, n=100, l=l, variant=M_().GEMM_AUTO)
-    _check_layer(g, ref, op, m, l)
+# Direct and staged gathers on both sides of where one takes over, in Init X (`x`) and the unmask (`u`): 48 / 49
+# entities with many tiles, 8190 / 8193 (entity, tile) pairs, one-level and two-level lists, ragged rows.
+@pytest.mark.parametrize("d,r,t,m,l,x,u", [
+    (3, (96, 64, 40), (8, 4), 6000, 48, True, False), (3, (96, 64, 40), (8, 4), 6000, 49, False, False),
+    (3, (96, 64, 40), (8, 4), 2730, 96, False, True), (3, (96, 64, 40), (8, 4), 2731, 96, False, False),
+    (2, (96, 40), (12,), 77, 33, True, True), (3, (100, 70, 36), (20, 16), 133, 95, True, True),
+    (3, (1536, 1024, 652), (80, 80), 65, 40, True, True), (3, (1536, 1024, 652), (80, 80), 31, 6, True, None)])
+def test_gathers_direct_and_staged(kernels, d, r, t, m, l, x, u):
+    out = []
+    names = kernels(lambda: out.extend(_run_layer(d, r, t, m=m, n=100, l=l, variant=M_().GEMM_AUTO)), by_role=True)
+    for role, direct in (("init_x", x), ("unmask", u)):
+        if direct is None:
+            assert names[role] == {"unmask_few"}
+        else:
+            assert ("dgather" in names[role], "pgather" in names[role]) == (direct, not direct), role
+    _check_layer(*out)
 
 
 # Segments that leave room for only 4, 2 or 1 staged rows a block (the gather of ranks above 1536 words),

@@ -8,6 +8,7 @@ import pytest
 
 import oracle as O
 from paper_2607_29221_gb300 import workloads as wl
+from test_drain_operands import drain_operands
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -83,6 +84,8 @@ def test_tc_random(Mm, N, K):
 @pytest.mark.parametrize("K", [256, 512, 1024, 768 + 32, 2048])
 @pytest.mark.parametrize("va,vb", [(ALL_M128, ALL_M128), (ALL_P127, ALL_M128), (ALL_P127, ALL_P127)])
 def test_tc_adversarial_digits(K, va, vb):
+    """The largest sums the groups reach (all their terms have one parity here;
+    test_tc_drain_points has the sums that would round)."""
     A = np.full((128, K), va, np.uint32)
     B = np.full((128, K), vb, np.uint32)
     assert np.array_equal(tc_gemm(A, B), ref(A, B))
@@ -316,11 +319,9 @@ def test_tc_few_tiles_split_k(Mm, N, K):
 def test_tc_drain_points(Mm, N, stages):
     """Every place of the two drains in a tile's last chunk (K of 1 to 45 stages
     of 32), one tile shared by CTAs and whole tiles one after another, with
-    all digits -128: a sum kept one stage too long leaves fp32's integers."""
+    operands whose sums leave fp32's integers when a pair of shift groups is
+    kept one stage too long (tests/test_drain_operands.py)."""
     for K in (32 * stages, 32 * stages - 27):
-        A = np.full((Mm, K), ALL_M128, np.uint32)
-        B = np.full((N, K), ALL_M128, np.uint32)
-        A[::3, ::5] = 0x01020304
-        B[::2, ::7] = 0xFEDCBA98
-        want = ref(A[:2], B[:2])[np.ix_(np.minimum(np.arange(Mm) % 3, 1), np.arange(N) % 2)]
+        A, B, S = drain_operands(Mm, N, K)
+        want = ref(A[:S], B[:S])[np.ix_(np.arange(Mm) % S, np.arange(N) % S)]
         assert np.array_equal(tc_gemm(A, B), want), K

@@ -126,7 +126,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     } else {
         uint32_t it = 0;
         bool ok = true;
-        const int rows = (a.br - warp + CWARPS - 1) / CWARPS;   // this warp's rows of a tile (0 for none)
+        // This warp's rows of a tile: RW or, for the last warps of a tile below BR rows, RW - 1 (and a row of zeros).
+        const int rows = (a.br - warp + CWARPS - 1) / CWARPS;
         for (int tile = blockIdx.x; ok && tile < a.tiles; tile += gridDim.x) {
             uint32_t acc[V];
 #pragma unroll
@@ -143,13 +144,13 @@ __global__ void __launch_bounds__(THREADS, 1)
                 uint4 b[RW];
 #pragma unroll
                 for (int r = 0; r < RW; ++r)
-                    b[r] = r < rows ? Bs[(warp + CWARPS * r) * (KC / 4) + lane] : make_uint4(0u, 0u, 0u, 0u);
+                    b[r] = r < RW - 1 || rows == RW ? Bs[(warp + CWARPS * r) * (KC / 4) + lane] : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
                 for (int t = 0; t < MT; ++t) {
                     const uint4 x = As[t * (KC / 4) + lane];
 #pragma unroll
                     for (int r = 0; r < RW; ++r)
-                        if (r < rows) acc[r * MT + t] += b[r].x * x.x + b[r].y * x.y + b[r].z * x.z + b[r].w * x.w;
+                        acc[r * MT + t] += b[r].x * x.x + b[r].y * x.y + b[r].z * x.z + b[r].w * x.w;
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&empty[s]);
@@ -238,10 +239,12 @@ mosaic_status launch_rw(const uint32_t *A, int64_t lda, const uint32_t *B, int64
     // fills them evenly: with tiles of 30 or 60 rows, 11404 rows left a sixth
     // of the last wave's SMs idle (x 8192, weights from HBM: 60.3 -> 58.1 us at
     // 1 token, 81.0 -> 76.0 at 8; x 32768: 215 -> 208 and 306 -> 286).  One
-    // wave keeps 30 or 60 rows: fewer and taller tiles read the token operand
-    // less often (7308 x 4096: 19.3 us either way).
+    // wave too: 60-row tiles on half of the SMs took 24.0 us at 8 tokens (5000 x
+    // 4096), 33-row tiles on all take 19.5.  At least 30 rows: fewer and taller
+    // tiles read the token operand less often.
     const int64_t waves = (N + 60 * (int64_t)sms - 1) / (60 * (int64_t)sms);
-    const int br = waves > 1 ? (int)((N + waves * sms - 1) / (waves * sms)) : N > 30 * (int64_t)sms ? 60 : 30;
+    const int64_t even = (N + waves * sms - 1) / (waves * sms);
+    const int br = even > 30 ? (int)even : 30;
     if (br <= 2 * CWARPS) return launch_skinny<MT, 2>(A, lda, B, ldb, Cm, ldc, Cin, ldcin, sgn, M, N, K, br, sms, st);
     if (br <= 3 * CWARPS) return launch_skinny<MT, 3>(A, lda, B, ldb, Cm, ldc, Cin, ldcin, sgn, M, N, K, br, sms, st);
     return launch_skinny<MT, 4>(A, lda, B, ldb, Cm, ldc, Cin, ldcin, sgn, M, N, K, br, sms, st);

@@ -288,11 +288,11 @@ def test_few_tokens_with_and_without_workspace(Mm, N, K):
 
 
 @pytest.mark.parametrize("Mm", [1, 3, 8, 11])
-@pytest.mark.parametrize("N", [4560, 4561, 9120, 9121, 11404, 18241])
+@pytest.mark.parametrize("N", [31, 4560, 4561, 6841, 7000, 9120, 9121, 11404, 18241])
 def test_few_tokens_tile_heights(Mm, N):
-    """One wave of 30- and 60-row tiles, and two or three waves of tiles cut to
-    fill them evenly (31 to 45 rows: some warps have a row less than others,
-    the last tile is ragged); no workspace, so the CUDA-core kernel runs."""
+    """One wave of 30-row tiles, and one to three waves of tiles cut to fill them
+    evenly (31 to 60 rows: some warps have a row less than others, the last tile
+    is ragged); no workspace, so the CUDA-core kernel runs."""
     M = _M()
     K = 260
     A = wl.uniform_u32(161 + Mm, Mm, K)

@@ -424,7 +424,7 @@ bool unmask_few_loses(int64_t l, int64_t m, int64_t rd, int nlev, const SparseLe
         if (m <= rows) return false;
         if (m <= 2 * rows) return rd > 2048 + 16 * sum_t;
         const int64_t rounds = (m + 4 * rows - 1) / (4 * rows);   // the last one may be nearly empty
-        return 2 * m > 9 * rows && m < 3 * rounds * rows && rd > 1792 + 4 * sum_t;
+        return 2 * m > (rd > 3072 ? 8 : 9) * rows && m < 3 * rounds * rows && rd > 1792 + 4 * sum_t;
     }
     if (!tiled) return false;
     if (m > 4 * rows) return rd + sum_t >= kFewRowWords;

@@ -90,6 +90,7 @@ def test_check_of_many_tokens(kernels, k, l, m, n, dz, clusters):
     (8, (2052,), (), 1, 0, 0, True), (5, (2052,), (), 1, 4, 0, False), (8, (2052,), (), 2, 0, 1, True),
     (8, (2048,), (), 2, 0, 0, True), (8, (2052,), (), 2, 4, 0, True), (8, (96, 2052), (40,), 2, 0, 0, True),
     (8, (1796,), (), 5, 0, 0, False), (8, (1792,), (), 5, 0, 0, True), (8, (1796,), (), 7, 0, 0, True),
+    (8, (3072,), (), 4, 4, 0, True), (8, (3076,), (), 4, 4, 0, False),
     (16, (1280,), (), 1, 0, 0, True), (9, (1284,), (), 1, 0, 0, False), (12, (848,), (), 1, 4, 0, True),
     (16, (856,), (), 2, 0, 0, False), (16, (64, 856), (4,), 2, 0, 0, True), (9, (1348,), (), 2, 4, 0, True),
     (16, (1352,), (), 2, 4, 0, False), (16, (64, 1352), (5,), 2, 4, 0, True)])

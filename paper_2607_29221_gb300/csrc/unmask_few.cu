@@ -18,14 +18,19 @@
 // lanes of four tokens each and a warp takes four rows at a time, which share
 // its dense reads of Q (unmask_rows_kernel).
 //
-// Measured on output rows x tokens, microseconds, against a streaming product,
-// a preparation and two gather passes:
-//             57344 x 1   57344 x 8  57344 x 16  8192 x 1  8192 x 8  8192 x 16
-//   before       82.7       113.2      139.4       15.6      33.8      38.5
-//   now          43.0        92.6      140.1        7.9      14.3      22.9
-// (43 us = 5.2 TB/s of L and S lists; at 16 tokens the shared-memory reads
-// and multiply-adds of a row bind instead: unmask_few_loses() tells where such a
-// call is better off with its rows on the tensor cores, 57344 x 16 in 104 us.)
+// Whole call on output rows x tokens, microseconds (ranks (1536, 1024, 652), t =
+// 80): the preparation, CUDA-core product and two gather passes that it replaced,
+// and one launch of this kernel; "flushed": L2 flushed before each call, events
+// around it, else back to back inside a CUDA graph, where 8192 rows of L and S
+// (33 MB) stay in L2:
+//                       57344 x 1   57344 x 8  57344 x 16   8192 x 1  8192 x 8  8192 x 16
+//   before, graph          81.9        113.2      139.2        14.8      33.7      38.3
+//   one launch, graph      42.6         94.6      140.0         7.5      14.0      22.6
+//   before, flushed        98.3        129.0      155.7        32.8      51.2      55.3
+//   one launch, flushed    55.3        106.5      149.5        16.4      28.7      38.9
+// (42.6 us = 5.2 TB/s of L and S lists; with more tokens the shared-memory reads
+// and multiply-adds of a row bind instead: unmask_few_loses() tells where a call
+// is better off on the general path, as 57344 x 16 is, 103 us in a graph.)
 #include "mosaic_internal.cuh"
 
 namespace mosaic {
@@ -386,8 +391,9 @@ bool unmask_few_ok(int64_t l, int64_t m, int64_t rd, int nlev, const SparseLevel
 // four rows a warp from 4865 rows on, 9728.  The lines were drawn through the
 // ratios one launch / general of r_d from 64 to 14000, one to three levels of t
 // = 8, 80, 128 and 400, and 16 to 57344 rows; the lists' words (sum_t = t_2 +
-// t_3) move a line up since the gathers then cost more.  Examples, whole call
-// inside a CUDA graph, one launch / general, microseconds:
+// t_3) move a line up since the gathers then cost more.  Examples, ratio of the
+// whole call inside a CUDA graph, one launch / general (with L2 flushed before
+// every call the ratios cross 1 at the same places):
 //   1 token, d = 1:  r_d 2048 x 57344 rows 1.00, 4096 x 4096 0.64, 4096 x 57344 1.18
 //   1 token, d = 3, t = 80:  4096 x 57344 0.99, 8192 x 8192 1.15
 //   4 tokens, d = 1:  8192 x 20480 1.14, 12000 x 2448 1.36, 12000 x 1024 0.69
@@ -397,13 +403,14 @@ bool unmask_few_ok(int64_t l, int64_t m, int64_t rd, int nlev, const SparseLevel
 //   16 tokens, d = 1:  1024 x 2400 0.64, 1536 x 16 1.20, 1536 x 2448 1.38, 2048 x 4864 1.44
 //   16 tokens, d = 3, t = 80:  1536 x 16 0.93, 2700 x 16 1.42, 1536 x 4096 1.08, 2700 x 2448 1.64
 // Beyond 9728 rows, 9 to 16 tokens stream L wherever a row holds enough words
-// (r_d + sum_t); whole call at 16 tokens, one launch -> streamed, microseconds,
-// by words a row:
+// (r_d + sum_t); whole call at 16 tokens, L2 flushed before each, events
+// around it (about 10 us of them are launch and events), one launch /
+// streamed, microseconds, by words a row:
 //   rows     812 (652, 80, 80)   1536 (one level)   732 (652, 80)   280 (200, 40, 40)
-//    8192      33.4 / 38.4          25.1 / 26.5       23.1 / 29.7      16.8 / 24.6
-//   10240      54.1 / 39.6          42.1 / 31.1       37.5 / 28.1      25.1 / 27.5
-//   20480      76.3 / 62.5          60.1 / 42.4       52.1 / 43.3      36.6 / 42.6
-//   57344     144.2 / 104.0        115.5 / 92.2       98.6 / 73.3      59.2 / 61.8
+//    8192      38.9 / 49.2          30.7 / 33.8       28.7 / 36.9      22.5 / 36.9
+//   10240      59.4 / 49.2          49.2 / 39.9       45.1 / 36.9      32.8 / 36.9
+//   20480      86.0 / 73.7          69.6 / 52.2       61.4 / 53.3      45.1 / 53.3
+//   57344     149.5 / 116.7        124.9 / 105.4      108.5 / 88.0     82.0 / 73.7
 constexpr int64_t kFewRowWords = 512;
 bool unmask_few_loses(int64_t l, int64_t m, int64_t rd, int nlev, const SparseLevel *lev) {
     int dev = 0;
@@ -428,8 +435,8 @@ bool unmask_few_loses(int64_t l, int64_t m, int64_t rd, int nlev, const SparseLe
     }
     if (!tiled) return false;
     if (m > 4 * rows) return rd + sum_t >= kFewRowWords;
-    if (m <= rows) return rd > 1280 + 5 * sum_t;
-    return rd > (m <= 2 * rows ? 850 : 1350) + 3 * sum_t;
+    if (m <= rows) return rd > (nlev || m < 128 ? 1280 : 1600) + 5 * sum_t;   // a few rows leave SMs idle
+    return rd > (m <= 2 * rows ? 850 : nlev ? 1350 : 1600) + 3 * sum_t;
 }
 
 mosaic_status unmask_few(int64_t l, int64_t m, const uint32_t *Z, int64_t ldz, int64_t dcol, int64_t rd,

@@ -91,9 +91,11 @@ def test_check_of_many_tokens(kernels, k, l, m, n, dz, clusters):
     (8, (2048,), (), 2, 0, 0, True), (8, (2052,), (), 2, 4, 0, True), (8, (96, 2052), (40,), 2, 0, 0, True),
     (8, (1796,), (), 5, 0, 0, False), (8, (1792,), (), 5, 0, 0, True), (8, (1796,), (), 7, 0, 0, True),
     (8, (3072,), (), 4, 4, 0, True), (8, (3076,), (), 4, 4, 0, False),
-    (16, (1280,), (), 1, 0, 0, True), (9, (1284,), (), 1, 0, 0, False), (12, (848,), (), 1, 4, 0, True),
-    (16, (856,), (), 2, 0, 0, False), (16, (64, 856), (4,), 2, 0, 0, True), (9, (1348,), (), 2, 4, 0, True),
-    (16, (1352,), (), 2, 4, 0, False), (16, (64, 1352), (5,), 2, 4, 0, True)])
+    (16, (1600,), (), 1, 0, 0, True), (9, (1604,), (), 1, 0, 0, False), (9, (1280,), (), 0, 124, 0, True),
+    (16, (1284,), (), 0, 124, 0, False), (16, (64, 1300), (4,), 1, 0, 0, True), (16, (64, 1304), (4,), 1, 0, 0, False),
+    (12, (848,), (), 1, 4, 0, True), (16, (856,), (), 2, 0, 0, False), (16, (64, 856), (4,), 2, 0, 0, True),
+    (9, (1600,), (), 2, 4, 0, True), (16, (1604,), (), 2, 4, 0, False), (16, (64, 1360), (4,), 2, 4, 0, True),
+    (16, (64, 1364), (4,), 2, 4, 0, False), (16, (64, 2000), (5,), 2, 4, 0, True)])
 def test_unmask_of_few_tokens(kernels, l, r, t, rounds, dm, pad, few):
     M = M_()
     m, d, S = rounds * 16 * sms() + dm, len(r), sum(r)

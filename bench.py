@@ -813,7 +813,7 @@ def run_decode_sweep(args, rank, world, torch, M, PR, proto, dev, stream, timed,
         del masks
         w_bytes = sum((ly.m + proto.sum_r) * ly.n_pad * 4 for ly in layers)
         # up to STREAMW_MAX_M tokens the server streams uint32 W' (4 B an element:
-        # CUDA cores up to SKINNY_MAX_M tokens, tensor cores above), beyond that
+        # CUDA cores up to 8 tokens, tensor cores from 9), beyond that
         # the tensor cores read its bf16 digit planes (8 B an element)
         skinny = variant != M.GEMM_IMAD and l <= M.SKINNY_MAX_M
         streamw = variant != M.GEMM_IMAD and M.SKINNY_MAX_M < l <= M.STREAMW_MAX_M

@@ -103,11 +103,17 @@ void count_launch();
 // set-up comes earlier, and no path returns earlier): that waits until all
 // earlier kernels have completed and their memory is visible, so the order
 // of the stream is kept and only the launch overlaps (2 to 3 us a launch
-// between back-to-back kernels).  It is for grids of at most one block per SM
-// (or of clusters): a grid of many small blocks would stack on the SMs that
-// free up first (the draws of a 301-token Init X went from 16 to 64 us), so
-// those are launched the ordinary way and only trigger.  What an earlier kernel
-// wrote is read with ordinary (coherent) or TMA loads, not __ldg.
+// between back-to-back kernels).  It is for persistent grids whose blocks all
+// fit on the device at once, and for the check's clusters: a grid of many
+// small blocks would stack on the SMs that free up first (the draws of a
+// 301-token Init X went from 16 to 64 us), so those are launched the ordinary
+// way and only trigger.  Grids of more than one block an SM can stack a little
+// too.  Early / ordinary: rotation and encode of 100 to 1300 rows of 16384 (two
+// blocks an SM, partly filled grids among them) 0.95 to 0.99 after another
+// kernel; the same kernel back to back 0.90 to 1.02, but 1.11 to 1.15 at 400
+// and 700 rows, where the one before ends unevenly.  The tiled gather of small
+// ranks (several blocks an SM) 0.98 to 1.02.  What an earlier kernel wrote is
+// read with ordinary (coherent) or TMA loads, not __ldg.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_enter() {
     asm volatile("griddepcontrol.wait;" ::: "memory");

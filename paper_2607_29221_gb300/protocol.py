@@ -171,9 +171,9 @@ class SecureLinear:
         """Untrusted accelerator: Z = X'_tm [W'; P]^T = [Y' | Q_1 .. Q_d] (token-major).
 
         Up to STREAMW_MAX_M tokens the product streams the uint32 W' (4 bytes an
-        element: CUDA cores up to SKINNY_MAX_M tokens, tensor cores with an
-        on-chip digit split above); more tokens run on the tensor cores from the
-        digit planes of W' and X'."""
+        element: CUDA cores up to 8 tokens, tensor cores with an on-chip digit
+        split from 9, where W' is not small); more tokens run on the tensor cores
+        from the digit planes of W' and X'."""
         l = Xp.shape[0]
         N = self.m + self.proto.sum_r
         Z = _u32(l, N, device=self.proto.device) if Z is None else Z

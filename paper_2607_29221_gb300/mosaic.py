@@ -177,9 +177,11 @@ def _stream(stream):
     if stream is not None:
         return stream if isinstance(stream, int) else stream.cuda_stream
     import torch
-    raw, device = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
-    if raw and device and torch.cuda.is_initialized():   # the raw handle, without a Stream object per call
-        return raw(device())
+    try:   # the raw handle, without a Stream object per call
+        if torch.cuda.is_initialized():
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    except AttributeError:   # a torch without these private accessors
+        pass
     return torch.cuda.current_stream().cuda_stream
 
 

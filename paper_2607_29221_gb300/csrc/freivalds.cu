@@ -50,6 +50,9 @@ __device__ __forceinline__ void dot_rows(uint32_t (&acc)[KV][T], const uint32_t 
         if (MINUS) acc[v][t] -= x * y;
         else acc[v][t] += x * y;
     };
+    // From 8 vectors on, the loads of four rows of A are in flight at once: one
+    // after another, their latencies made up most of a share.
+    constexpr int G = KV >= 8 ? 4 : 1;
     int64_t c = c0;
     if (vec) {   // 16-byte loads; c0 is a multiple of 4
         const int64_t quads = (c1 - c0) >> 2;
@@ -59,9 +62,6 @@ __device__ __forceinline__ void dot_rows(uint32_t (&acc)[KV][T], const uint32_t 
 #pragma unroll
             for (int t = 0; t < T; t++)
                 x[t] = t < tn ? __ldcg(reinterpret_cast<const uint4 *>(B + t * ldb + c0) + i) : make_uint4(0u, 0u, 0u, 0u);
-            // From 8 vectors on, the loads of four rows of A are in flight at once: one
-            // after another, their latencies made up most of a share.
-            constexpr int G = KV >= 8 ? 4 : 1;
 #pragma unroll
             for (int v0 = 0; v0 < KV; v0 += G) {
                 if (v0 >= k) break;
@@ -88,11 +88,15 @@ __device__ __forceinline__ void dot_rows(uint32_t (&acc)[KV][T], const uint32_t 
 #pragma unroll
         for (int t = 0; t < T; t++) x[t] = t < tn ? __ldcg(B + t * ldb + i) : 0u;
 #pragma unroll
-        for (int v = 0; v < KV; v++) {
-            if (v >= k) break;
-            const uint32_t y = __ldca(A + v * lda + i);
+        for (int v0 = 0; v0 < KV; v0 += G) {
+            if (v0 >= k) break;
+            uint32_t y[G];
 #pragma unroll
-            for (int t = 0; t < T; t++) mac(v, t, y, x[t]);
+            for (int g = 0; g < G; g++) y[g] = G == 1 || v0 + g < k ? __ldca(A + (v0 + g) * lda + i) : 0u;
+#pragma unroll
+            for (int g = 0; g < G; g++)
+#pragma unroll
+                for (int t = 0; t < T; t++) mac(v0 + g, t, y[g], x[t]);
         }
     }
 }
@@ -109,7 +113,7 @@ __device__ __forceinline__ void dot_rows(uint32_t (&acc)[KV][T], const uint32_t 
 // products on 18 blocks each and a comparison took 18.1 + 17.9 + 2.0 us.
 constexpr int kChkThreads = 256;
 template <int KV, int T>
-__global__ void __launch_bounds__(kChkThreads, KV >= 8 ? 2 : 4)
+__global__ void __launch_bounds__(kChkThreads, KV >= 8 && T > 1 ? 2 : 4)
     check_kernel(int k, const uint32_t *a, const uint32_t *Ychk, int64_t m, int64_t n_pad, int64_t l,
                  const uint32_t *Z, int64_t ldz, const uint32_t *Xp, int64_t ldx, uint32_t *bad, uint32_t *n_bad,
                  int vec_z, int vec_x) {

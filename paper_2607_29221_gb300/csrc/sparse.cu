@@ -579,8 +579,9 @@ mosaic_status launch_pgather(const GatherArgs &a, cudaStream_t st) {
 // SMs).  Up to kDirectTasks pairs, warps take two: that still pays with two levels
 // of short lists (one launch and one pass over the outputs less) or very short
 // ones.  With the entities as output rows (Init X) it is also taken up to
-// kDirectEnts entities whatever the tiles, or kDirectEntsPadded where the staged
-// gather's rounds of 16 pairs hold at least a quarter of padding.  Direct /
+// kDirectEnts entities whatever the tiles, kDirectEntsFull where every list is
+// one nearly full round of the staged gather (16 pairs) and there are more
+// than kDirectEntsTasks pairs.  Direct /
 // staged, whole call inside a CUDA graph, m outputs, l tokens, by (ranks) and t:
 //                     (1536, 1024, 652)               (512, 64)
 //   t                4    16    80   160   400      4    16    80   160
@@ -593,10 +594,14 @@ mosaic_status launch_pgather(const GatherArgs &a, cudaStream_t st) {
 //   Init X of 8192 + 57344 rows
 //   l = 40         0.59  0.89  0.91  0.87  0.80   0.63  1.10  0.81  0.76
 //   l = 48         0.63  0.99  1.01  0.97  0.91   0.70  1.24  0.91  0.89
-//   and l = 48 at t = 12 / 20 / 24 / 32:  0.87 0.77 0.85 1.03, (512, 64) 1.09 0.82 0.94 1.12
+//   l = 48 at t = 12, 20, 24, 32:  0.87 0.77 0.85 1.03, (512, 64) 1.09 0.82 0.94 1.12
+//   l = 44 at t = 16, 32, 80:      0.93 0.98 0.96, (512, 64) 1.16 1.06 0.86
+//   Init X of 4096 + 4096 / 8192 + 8192 rows (12288 / 24576 pairs), l = 48
+//   4096           0.65  0.84  0.93     -  0.90      -  1.01  0.94     -
+//   8192           0.60  0.94  0.95     -  0.90      -  1.03  0.90     -
 // ---------------------------------------------------------------------------
 constexpr int kDgWarps = 32;
-constexpr int64_t kDirectTasks = 8192, kDirectEnts = 40, kDirectEntsPadded = 48;
+constexpr int64_t kDirectTasks = 8192, kDirectEnts = 48, kDirectEntsFull = 40, kDirectEntsTasks = 32768;
 
 struct DirectArgs {
     const uint32_t *img[2], *img2[2];   // per level: images of the first and the second job
@@ -708,7 +713,8 @@ bool direct_ok(bool list_is_col, int64_t tiles, int64_t nlist, const SparseLevel
     const int64_t tasks = tiles * nlist;
     if (tasks <= (int64_t)sm_count(dev) * kDgWarps) return true;
     if (tasks <= kDirectTasks && longest <= (nlev == 2 ? 80 : 8)) return true;
-    return !list_is_col && nlist <= (4 * pairs <= 3 * 16 * rounds ? kDirectEntsPadded : kDirectEnts);
+    const bool full_round = longest <= 16 && 4 * pairs > 3 * 16 * rounds;
+    return !list_is_col && nlist <= (full_round && tasks > kDirectEntsTasks ? kDirectEntsFull : kDirectEnts);
 }
 
 void direct_levels(DirectArgs &d, const SparseLevel *lev, int nlev) {

@@ -124,8 +124,10 @@ def test_unmask_of_few_tokens(kernels, l, r, t, rounds, dm, pad, few):
     ((96, 64, 40), (8, 4), 1024, 1056, 126, True), ((96, 64, 40), (8, 4), 1024, 1056, 127, False),
     ((200, 180, 40), (80, 84), 1024, 1408, 64, True), ((200, 180, 40), (80, 84), 1024, 1408, 65, False),
     ((64, 40), (12,), 512, 1920, 64, True), ((64, 40), (12,), 512, 1920, 65, False), ((64, 40), (8,), 512, 1920, 65, True),
-    ((64, 40), (12,), 8192, 6000, 48, True), ((64, 40), (12,), 8192, 6000, 49, False),
-    ((64, 40), (16,), 8192, 6000, 40, True), ((64, 40), (16,), 8192, 6000, 41, False)])
+    ((64, 40), (12,), 8192, 20000, 48, True), ((64, 40), (12,), 8192, 20000, 49, False),
+    ((64, 40), (16,), 8192, 20000, 40, True), ((64, 40), (16,), 8192, 20000, 41, False),
+    ((256, 40), (32,), 8192, 20000, 48, True), ((64, 40), (16,), 8192, 13632, 48, True),
+    ((64, 40), (16,), 8192, 13696, 48, False), ((64, 40), (16,), 8192, 13632, 49, False)])
 def test_init_x_gathers(kernels, r, t, n_pad, m, l, direct):
     M = M_()
     p, S = M.default_params(d=len(r), r=r, t=(0,) + t), sum(r)

@@ -63,7 +63,8 @@ struct GatherArgs {
     uint32_t *out2;
 };
 
-// Staged rows plus the per-warp list rings.
+// Staged rows plus the per-warp list rings; at most kGatherSmem bytes.
+constexpr size_t kGatherSmem = 220 * 1024;
 constexpr size_t gather_smem(int tg, int64_t segp) {
     return ((size_t)tg * (size_t)segp + 3) / 4 * 4 * sizeof(uint32_t) +
            (size_t)GW * kRing * (32 / tg) * 32 * sizeof(uint32_t);
@@ -829,10 +830,9 @@ mosaic_status launch_few(const GatherArgs &a, cudaStream_t st) {
 template <int TG, bool LIST_IS_COL, bool CLAMP>
 mosaic_status launch_gather(const GatherArgs &a, cudaStream_t st) {
     const size_t smem = gather_smem(TG, a.segp);
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(gather_kernel<TG, LIST_IS_COL, CLAMP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) != cudaSuccess)
-        return MOSAIC_ERR_CUDA;
+    // One limit for every call: a limit per call could be lowered by another thread before this launch.
+    static std::atomic<unsigned long long> attr_set{0};   // one bit per device ordinal
+    if (!ensure_smem_limit(attr_set, gather_kernel<TG, LIST_IS_COL, CLAMP>, kGatherSmem)) return MOSAIC_ERR_CUDA;
     dim3 grid((unsigned)((a.nlist + G_ENTS - 1) / G_ENTS), (unsigned)((a.g_count + TG - 1) / TG));
     if (grid.y > 65535) return MOSAIC_ERR_SHAPE;
     {
@@ -855,7 +855,7 @@ mosaic_status dispatch_gather(GatherArgs a, cudaStream_t st) {
     a.segp = (int64_t)(a.r + 31) / 32 * 32 + 1;
     // The largest row tile with which two CTAs fit on an SM (one CTA stages
     // while the other gathers); else the largest that fits at all.
-    const size_t two = 113 * 1024, one = 220 * 1024;
+    const size_t two = 113 * 1024, one = kGatherSmem;
     for (size_t cap : {two, one}) {
         if (gather_smem(32, a.segp) <= cap) return launch_gather<32, LIST_IS_COL, CLAMP>(a, st);
         if (gather_smem(16, a.segp) <= cap) return launch_gather<16, LIST_IS_COL, CLAMP>(a, st);

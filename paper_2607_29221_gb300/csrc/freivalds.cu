@@ -206,8 +206,8 @@ int check_resident(int dev, int s) {
 // / products, by k vectors, l tokens and m = n_pad:
 //   m        4, 2048     4, 4096     8, 1024     8, 2048     8, 4096    16, 4096
 //   64      5.1 /  4.8  9.7 /  5.0  5.0 /  5.7   10 /  5.8       -           -
-//   1024    7.0 /  8.7   12 /  9.0  5.9 / 11.7   11 / 11.8   22 / 12.1       -
-//   8192     37 / 38.7   74 / 51.1   19 / 56.5   43 / 58.3   88 / 61.3  151 / 98.6
+//   1024    7.0 /  8.7   12 /  8.7  5.9 / 11.7   11 / 11.8   22 / 11.7       -
+//   8192     37 / 38.7   74 / 50.6   19 / 56.5   43 / 58.3   88 / 58.1  151 / 96.9
 template <int KV, int T>
 mosaic_status launch_check(int k, const uint32_t *a, const uint32_t *Ychk, int64_t m, int64_t n_pad, int64_t l,
                            const uint32_t *Z, int64_t ldz, const uint32_t *Xp, int64_t ldx, uint32_t *bad,
